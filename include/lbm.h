@@ -161,8 +161,9 @@ lbm_status lbm_init_phi(lbm_ctx* ctx, const double* phi, const double* u, const 
 lbm_status lbm_set_velocity(lbm_ctx* ctx, int kind, double U, double period);
 
 /* Advance n >= 0 time steps (Eqs. 4 and 20: stream, then collide in moment space with
- * Eqs. 17-18 and 31-32).  Asynchronous on the context's stream.  Pairs of steps are
- * replayed from CUDA graphs captured on first use (see LBM_TUNE_GRAPHS). */
+ * Eqs. 17-18 and 31-32).  Asynchronous on the context's stream.  Small grids take all n
+ * steps in one kernel (see LBM_TUNE_BRICKS); on others pairs of steps are replayed from
+ * CUDA graphs captured on first use (see LBM_TUNE_GRAPHS). */
 lbm_status lbm_step(lbm_ctx* ctx, int n);
 
 /* Macroscopic fields at the current time, computed on the device from the current
@@ -283,6 +284,15 @@ lbm_status lbm_write_state(lbm_ctx* ctx, const float* f, const float* g,
  * value per cell; its wait for the copies is bounded like the chemical-potential pass's
  * (LBM_TUNE_TMA_WAIT_POLLS, same error reporting).  lbm_get_tuning reports 1 only while
  * it applies.  Identical results.
+ * LBM_TUNE_BRICKS: 1 (default) lets lbm_step and lbm_step_reduce advance small grids
+ * (LBM_PATTERN_AB; up to 640,000 cells, 180,000 with 16-bit populations, 1.6 million in
+ * interface-tracking mode) by one kernel per call that keeps every block on its own brick of
+ * cells for all the steps, blocks waiting for their neighbours between steps.  The wait is
+ * bounded; one that runs out is reported as LBM_ETIMEOUT like the TMA passes' waits.
+ * lbm_get_tuning reports 1 only while it applies: not while profiling, not while one of the
+ * parameters that choose among the three-kernel step's passes (MU_TMA, GRAPHS, ROWS,
+ * CELL_PAIRS, STENCIL_STAGE, FUSED, or a poll budget other than the default) is set to
+ * anything but its default, and not on a stream under capture.  Identical results.
  * Setting any parameter drops the captured graphs (and waits for the context's
  * stream).
  * lbm_set_tuning returns LBM_EINVAL for an unknown parameter or a value out of range. */
@@ -298,6 +308,7 @@ lbm_status lbm_write_state(lbm_ctx* ctx, const float* f, const float* g,
 #define LBM_TUNE_CELL_PAIRS 9
 #define LBM_TUNE_STENCIL_STAGE 10
 #define LBM_TUNE_PREFETCH_COLLIDE_SUMS 11
+#define LBM_TUNE_BRICKS 12
 lbm_status lbm_set_tuning(lbm_ctx* ctx, int param, int value);
 lbm_status lbm_get_tuning(const lbm_ctx* ctx, int param, int* value);
 

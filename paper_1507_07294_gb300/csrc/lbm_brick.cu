@@ -1,0 +1,184 @@
+// Plan and launch of the resident-brick kernel (lbm_brick.cuh).
+#include <algorithm>
+
+#include "lbm_internal.h"
+
+namespace lbm {
+
+const void* brick_kernel_f32(int mode, int var, bool pair);
+cudaError_t state_sums_f32(const float* state, const float* phi, const Geometry& geo, double* partial,
+                        double* out, int* count, cudaStream_t st);
+const void* brick_kernel_f16(int mode, int var, bool pair);
+cudaError_t state_sums_f16(const float* state, const float* phi, const Geometry& geo, double* partial,
+                        double* out, int* count, cudaStream_t st);
+const void* brick_kernel_bf16(int mode, int var, bool pair);
+cudaError_t state_sums_bf16(const float* state, const float* phi, const Geometry& geo, double* partial,
+                        double* out, int* count, cudaStream_t st);
+
+namespace {
+
+// ceil(2^kBrickDivShift / d), and whether k * it >> kBrickDivShift = k / d for every k up to
+// `most`.
+unsigned brick_div(int d) { return ((1u << kBrickDivShift) + d - 1) / d; }
+
+bool brick_div_ok(int d, long long most) {
+  const unsigned long long m = brick_div(d), over = m * d - (1ull << kBrickDivShift);
+  return most * m < (1ull << 32) && most * over < (1ull << kBrickDivShift);
+}
+
+const void* kernel_of(const Geometry& geo, const Physics& ph, int mode, bool pair) {
+  const int var = mode == kBrickTracking
+                      ? 0
+                      : (ph.srt_flow ? kVarSrtFlow : 0) | (ph.d3q7_stencil ? kVarD3Q7 : 0);
+  return geo.storage == kF16    ? brick_kernel_f16(mode, var, pair)
+         : geo.storage == kBF16 ? brick_kernel_bf16(mode, var, pair)
+                                : brick_kernel_f32(mode, var, pair);
+}
+
+// One way to cut an axis: bricks, cells of the largest, bricks within the cells a step reads.
+struct AxisCut {
+  int nb, b, reach;
+};
+
+AxisCut cut_axis(int n, int want, int halo) {
+  AxisCut c;
+  c.nb = (n + want - 1) / want;
+  c.b = (n + c.nb - 1) / c.nb;
+  const int least = n / c.nb;
+  c.reach = (halo + 1 + least - 1) / least;
+  return c;
+}
+
+// Whether the kernel's small divisions are exact for bricks of these sizes (cell numbers run
+// up to two rounds of threads beyond a brick's cells).
+bool divisions_ok(const AxisCut c[3], int halo) {
+  const long long cells = static_cast<long long>(c[0].b) * c[1].b * c[2].b + 2 * kBrickThreads;
+  if (!brick_div_ok(c[0].b, cells) || !brick_div_ok(c[1].b, cells / c[0].b + 1)) return false;
+  for (int add : {2, 2 * halo, 2 * halo + 2}) {
+    const long long x = c[0].b + add, y = c[1].b + add, z = c[2].b + add;
+    if (!brick_div_ok(static_cast<int>(x), x * y * z) || !brick_div_ok(static_cast<int>(y), y * z + 1))
+      return false;
+  }
+  return true;
+}
+
+}  // namespace
+
+// The line lies where the two state arrays outgrow the L2 cache (129 MB): 640,000 cells of
+// 2 x 100 B coupled in FP32, 1.6M of 2 x 40 B in tracking mode, where f and phi u are all
+// that moves.  Measured just inside it: 96x96x64 (590k cells) 32.8 -> 28.1 us a step,
+// tracking at 116^3 (1.56M) 49.3 -> 32.9 us; beyond it (64x64x256, 1.05M cells) the bricks'
+// halos come from DRAM and the kernel takes 57-63 us where the three passes take 63.7.
+// With 16-bit populations the coupled kernel gains less (its 2-byte loads bring half as much
+// each) and the line is where it stops gaining: 56x57x55 (176k cells) 19.5 -> 13.9 us,
+// 64^3 (262k) 18.4 -> 18.5.
+long long brick_most_cells(int mode, int storage) {
+  if (mode == kBrickTracking) return 1600000;
+  return storage == kF32 ? 640000 : 180000;
+}
+
+// The cut with the least modelled step time among those that keep every block resident.  The
+// model, fitted to 190 measured cuts of 16^3 to 96x96x64 (within 20 % of them): 3.65 us for
+// the wait, the loads' latency and the stores, and per block of an SM 0.44 ns for each place
+// of its phi and mu regions and 2.7 ns (tracking: 1.2) for each of its cells in whole rounds
+// of threads, more for short rows (a region row of 20 touches as many lines as one of 36) and
+// for rows that do not start on tiles; a lone block with several rounds per SM waits more.
+// Two cells per thread pay from about 1024 cells a block (64x64x128, 256 bricks of 32x8x8:
+// 24.9 us, one cell per thread 26.3); they leave room for 2 blocks an SM instead of 3.
+// Measured per step, three passes -> bricks: 16^3 12.3 -> 4.2 us, 32^3 14.3 -> 5.1,
+// 48^3 16.4 -> 7.9, 64^3 24.6 -> 13.9, 64x64x128 38.9 -> 25.1, 37x41x45 15.4 -> 8.5;
+// tracking 32^3 19.5 -> 3.8, 64^3 18.5 -> 8.0, 100^3 38.2 -> 21.3; FP16 32^3 14.4 -> 6.2.
+BrickPlan brick_plan(const Geometry& geo, const Physics& ph, int mode, int sms) {
+  BrickPlan p{};
+  if (geo.n > brick_most_cells(mode, geo.storage) || sms < 1) return p;
+  const int halo = mode == kBrickTracking ? 1 : 2;
+  constexpr int kWant = 9;
+  static const int want[2][kWant] = {{8, 12, 16, 24, 32, 48, 64, 96, 128}, {2, 3, 4, 5, 6, 8, 10, 12, 16}};
+  AxisCut axis[3][kWant];
+  for (int i = 0; i < kWant; ++i) {
+    axis[0][i] = cut_axis(geo.nx, want[0][i], halo);
+    axis[1][i] = cut_axis(geo.ny, want[1][i], halo);
+    axis[2][i] = cut_axis(geo.nz, want[1][i], halo);
+  }
+  double cost = 0.0;
+  for (int i = 0; i < kWant; ++i)
+    for (int j = 0; j < kWant; ++j)
+      for (int k = 0; k < kWant; ++k) {
+        const AxisCut c[3] = {axis[0][i], axis[1][j], axis[2][k]};
+        const long long bricks = static_cast<long long>(c[0].nb) * c[1].nb * c[2].nb;
+        if (bricks > 3LL * sms || bricks > kBrickMax) continue;
+        long long cells = 1, phi = 1, mu = 1, offsets = 1, around = 1;
+        for (const AxisCut& a : c) {
+          cells *= a.b;
+          phi *= a.b + 2 * halo;
+          mu *= a.b + 2;
+          offsets *= a.b + 2 * halo + 2;
+          around *= std::min(a.nb, 2 * a.reach + 1);
+        }
+        if (mode == kBrickTracking) mu = 0;
+        const long long smem = 4 * (phi + mu + offsets);
+        const int per = static_cast<int>((bricks + sms - 1) / sms);
+        if (around > kBrickThreads || smem > kBrickSmem || per * (smem + 1024) > 226 * 1024) continue;
+        for (int pair = 0; pair < 2; ++pair) {
+          if (pair && (mode == kBrickTracking || cells < 1024 || per > 2)) continue;
+          const long long round = pair ? 2 * kBrickThreads : kBrickThreads;
+          const double cell = mode == kBrickTracking ? 1.2e-3 : (cells >= 1024 && !pair ? 2.9e-3 : 2.7e-3);
+          double work = 4.4e-4 * (phi + mu) + cell * ((cells + round - 1) / round * round);
+          work *= 1.0 + 4.0 / c[0].b;
+          if (geo.row_tiles && c[0].b % 16 != 0) work *= 1.08;
+          const double est = 3.65 + per * work * (per == 1 && cells > 512 ? 1.3 : 1.0);
+          if ((p.nbricks && est >= cost) || !divisions_ok(c, halo)) continue;
+          cost = est;
+          p.nbricks = static_cast<int>(bricks);
+          p.mode = mode;
+          p.pair = pair;
+          p.around = static_cast<int>(around);
+          p.smem = static_cast<int>(smem);
+          for (int a = 0; a < 3; ++a) {
+            p.nb[a] = c[a].nb;
+            p.b[a] = c[a].b;
+            p.reach[a] = c[a].reach;
+          }
+        }
+      }
+  if (p.nbricks == 0) return p;
+  const void* k = kernel_of(geo, ph, mode, p.pair != 0);
+  int per = 0;
+  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kBrickSmem) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, kBrickThreads, p.smem) != cudaSuccess ||
+      static_cast<long long>(per) * sms < p.nbricks) {
+    cudaGetLastError();
+    return BrickPlan{};
+  }
+  p.m_qx = brick_div(p.b[0] + 2 * halo + 2);
+  p.m_qy = brick_div(p.b[1] + 2 * halo + 2);
+  p.m_px = brick_div(p.b[0] + 2 * halo);
+  p.m_py = brick_div(p.b[1] + 2 * halo);
+  p.m_mx = brick_div(p.b[0] + 2);
+  p.m_my = brick_div(p.b[1] + 2);
+  p.m_bx = brick_div(p.b[0]);
+  p.m_by = brick_div(p.b[1]);
+  return p;
+}
+
+cudaError_t launch_brick(float* state0, float* state1, float* phi, const Geometry& geo,
+                         const Physics& ph, const BrickPlan& plan, const BrickTimes& times, int steps,
+                         int* flags, int base, bool have_prev, int* err, long long polls,
+                         cudaStream_t st) {
+  BrickPlan bp = plan;
+  bp.steps = steps;
+  int hp = have_prev ? 1 : 0;
+  void* args[] = {&state0, &state1, &phi, const_cast<Geometry*>(&geo), const_cast<Physics*>(&ph), &bp,
+                  const_cast<BrickTimes*>(&times), &flags, &base, &hp, &err, &polls};
+  return cudaLaunchCooperativeKernel(kernel_of(geo, ph, plan.mode, plan.pair != 0), dim3(plan.nbricks),
+                                     dim3(kBrickThreads), args, plan.smem, st);
+}
+
+cudaError_t launch_state_sums(const float* state, const float* phi, const Geometry& geo, double* partial,
+                              double* out, int* count, cudaStream_t st) {
+  return geo.storage == kF16    ? state_sums_f16(state, phi, geo, partial, out, count, st)
+         : geo.storage == kBF16 ? state_sums_bf16(state, phi, geo, partial, out, count, st)
+                                : state_sums_f32(state, phi, geo, partial, out, count, st);
+}
+
+}  // namespace lbm

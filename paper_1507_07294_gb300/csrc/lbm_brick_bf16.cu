@@ -1,0 +1,13 @@
+// The resident-brick kernel (lbm_brick.cuh) for BF16 populations.
+#include "lbm_brick.cuh"
+
+namespace lbm {
+
+const void* brick_kernel_bf16(int mode, int var, bool pair) { return brick_kernel<kBF16>(mode, var, pair); }
+
+cudaError_t state_sums_bf16(const float* state, const float* phi, const Geometry& geo, double* partial,
+                           double* out, int* count, cudaStream_t st) {
+  return state_sums<kBF16>(state, phi, geo, partial, out, count, st);
+}
+
+}  // namespace lbm

@@ -1,0 +1,13 @@
+// The resident-brick kernel (lbm_brick.cuh) for FP16 populations.
+#include "lbm_brick.cuh"
+
+namespace lbm {
+
+const void* brick_kernel_f16(int mode, int var, bool pair) { return brick_kernel<kF16>(mode, var, pair); }
+
+cudaError_t state_sums_f16(const float* state, const float* phi, const Geometry& geo, double* partial,
+                           double* out, int* count, cudaStream_t st) {
+  return state_sums<kF16>(state, phi, geo, partial, out, count, st);
+}
+
+}  // namespace lbm

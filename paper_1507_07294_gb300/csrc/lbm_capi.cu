@@ -53,6 +53,7 @@ struct lbm_ctx {
   long long tma_polls = -1;  // poll budget of the copy's wait; -1: the kernel default
   int row_tiles = 0;         // Geometry::row_tiles when LBM_TUNE_ROWS is on
   int pairs = 0;             // Geometry::pairs when LBM_TUNE_CELL_PAIRS is on
+  int default_stage = 0;     // Geometry::stage as lbm_create set it
   int stage_rows = 0;        // Geometry::stage when LBM_TUNE_STENCIL_STAGE is on
   int prefetch_sums = 0;     // Geometry::prefetch_collide of the steps that sum their result
 
@@ -62,6 +63,14 @@ struct lbm_ctx {
   int fused_seg = 0;
   int fused_pf = 0;
   int sms = 0;
+
+  // resident-brick steps of small grids (lbm_brick.cuh): the plan (none: nbricks 0), the
+  // bricks' step counters and what they hold now; `brick_reset`: clear them first
+  lbm::BrickPlan brick{};
+  int* brick_flags = nullptr;
+  int brick_base = 0;
+  bool brick_reset = true;
+  bool use_bricks = true;
 
   // CUDA graphs of two consecutive steps, one per parity of the stored state (which
   // array is current, or the AA step parity, and which phi array is current), replayed
@@ -219,9 +228,11 @@ void release(lbm_ctx* c) {
   dev_free(c, c->partial);
   dev_free(c, c->red);
   dev_free(c, c->step_parts);
+  dev_free(c, c->brick_flags);
   c->pop[0] = c->pop[1] = c->phi = c->phi_buf[0] = c->phi_buf[1] = c->mu = c->stage = nullptr;
   c->partial = c->red = nullptr;
   c->step_parts = nullptr;
+  c->brick_flags = nullptr;
 }
 
 // Device error word (1: a bounded wait on a TMA copy ran out), kept in red[7].
@@ -237,6 +248,7 @@ lbm_status take_device_error(lbm_ctx* c, const double* h) {
   std::memcpy(&word, h + 7, sizeof(word));
   if (word == 0) return LBM_OK;
   cudaMemsetAsync(c->red + 7, 0, sizeof(double), c->stream);
+  c->brick_reset = true;  // blocks that gave up did not count their steps
   if (word >= 2) {
     c->retired = true;
     return fail(c, LBM_ECUDA,
@@ -244,8 +256,8 @@ lbm_status take_device_error(lbm_ctx* c, const double* h) {
                 "returned; the context is retired (destroy it)");
   }
   return fail(c, LBM_ETIMEOUT,
-              "a bounded wait for a TMA copy in the chemical-potential pass ran out; the "
-              "affected steps are not valid");
+              "a bounded wait for a TMA copy of the three-kernel step, or of one brick of a small "
+              "grid for another, ran out; the affected steps are not valid");
 }
 
 // Refuses launches on a context that is not initialised or has been retired.
@@ -535,6 +547,74 @@ lbm_status capture_pair(lbm_ctx* c, int parity) {
   return LBM_OK;
 }
 
+size_t brick_flag_bytes() {
+  return (static_cast<size_t>(lbm::kBrickMax) * lbm::kBrickFlag + 8) * sizeof(int);
+}
+
+// Whether the next n steps go through the resident-brick kernel.  The parameters that
+// choose among the passes of the three-kernel step select that step when set to anything
+// but their defaults, and so does an explicit poll budget (it bounds those passes' copies).
+// A stream under capture takes the three-kernel step too: a replayed launch would find the
+// step counters of its first run.
+bool brick_applies(const lbm_ctx* c, int n) {
+  if (!(c->use_bricks && c->brick.nbricks > 0 && n > 0 && !c->profiling && c->use_graphs &&
+        !fused_applies(c) && c->geo.row_tiles == c->row_tiles && c->geo.pairs == c->pairs &&
+        c->geo.stage == c->default_stage && c->use_phi_map &&
+        (c->tma_polls < 0 || c->tma_polls == lbm::mu_tma_default_polls())))
+    return false;
+  // with 16-bit storage the first step reads the phi array that the last one writes
+  if (n == 1 && c->geo.storage != lbm::kF32) return false;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(c->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+}
+
+// n steps through the resident-brick kernel; with sums_out the sums of the state after them.
+lbm_status brick_steps(lbm_ctx* c, int n, double* sums_out) {
+  const bool tracking = c->vel_kind != LBM_VELOCITY_NONE;
+  while (n > 0) {
+    const int most = tracking ? lbm::kBrickTrackSteps : lbm::kBrickSteps;
+    int k = n < most ? n : most;
+    if (n - k == 1) --k;  // a single last step could not go this way with 16-bit storage
+    if (c->brick_reset || c->brick_base > (1 << 30)) {
+      LBM_CK(c, cudaMemsetAsync(c->brick_flags, 0, brick_flag_bytes(), c->stream));
+      c->brick_base = 0;
+      c->brick_reset = false;
+    }
+    lbm::BrickTimes times;
+    for (int i = 0; i < lbm::kBrickTrackSteps; ++i)
+      times.tf[i] = tracking && i < k ? velocity_time_factor(c, c->step + i) : 1.0f;
+    const cudaError_t e = lbm::launch_brick(
+        c->pop[c->cur], c->pop[1 - c->cur], c->phi, c->geo, c->ph, c->brick, times, k,
+        c->brick_flags, c->brick_base, c->have_prev, error_word(c), lbm::mu_tma_default_polls(),
+        c->stream);
+    if (e == cudaErrorCooperativeLaunchTooLarge) {
+      // fewer SMs than the device has (a partition of it): the three-kernel step from here on
+      cudaGetLastError();
+      c->brick = lbm::BrickPlan{};
+      return sums_out ? lbm_step_reduce_async(c, n, sums_out) : lbm_step(c, n);
+    }
+    LBM_CK(c, e);
+    c->brick_base += k;
+    c->cur = (c->cur + k) & 1;
+    c->have_prev = true;
+    c->step += k;
+    n -= k;
+  }
+  if (sums_out)
+    LBM_CK(c, lbm::launch_state_sums(c->pop[c->cur], c->phi, c->geo, c->partial, sums_out,
+                                     c->brick_flags + lbm::kBrickMax * lbm::kBrickFlag, c->stream));
+  return LBM_OK;
+}
+
+// The plan for the context's mode (coupled or tracking).
+void plan_bricks(lbm_ctx* c) {
+  c->brick = lbm::BrickPlan{};
+  if (c->params.pattern == LBM_PATTERN_AB)
+    c->brick = lbm::brick_plan(
+        c->geo, c->ph, c->vel_kind == LBM_VELOCITY_NONE ? lbm::kBrickCoupled : lbm::kBrickTracking,
+        c->sms);
+}
+
 // Whether the last step of lbm_step_reduce can carry the sums (else a separate pass).
 bool fused_sums(const lbm_ctx* c) {
   return c->vel_kind == LBM_VELOCITY_NONE &&
@@ -585,7 +665,7 @@ lbm_status lbm_create(const lbm_grid* grid, const lbm_params* params, const lbm_
   if (c->pairs && lbm::stage_shape_ok(c->geo)) c->stage_rows = 1;
   // on by default with FP32 populations only: with 16-bit ones the pass is faster
   // loading its stencils per cell (the block waits for all its rows before computing)
-  c->geo.stage = params->storage == LBM_STORAGE_FP32 ? c->stage_rows : 0;
+  c->geo.stage = c->default_stage = params->storage == LBM_STORAGE_FP32 ? c->stage_rows : 0;
   // L2 prefetch distances: one wave of resident blocks
   {
     int dev = 0, sms = 0;
@@ -618,9 +698,12 @@ lbm_status lbm_create(const lbm_grid* grid, const lbm_params* params, const lbm_
   c->partial = static_cast<double*>(dev_alloc(c, sizeof(double) * 5 * lbm::kReduceMaxParts));
   c->red = static_cast<double*>(dev_alloc(c, sizeof(double) * 8));
   c->step_parts = static_cast<float*>(dev_alloc(c, step_parts_bytes(c->geo.n)));
+  plan_bricks(c);
+  c->brick_flags = static_cast<int*>(dev_alloc(c, brick_flag_bytes()));
   if (!c->pop[0] || (params->pattern == LBM_PATTERN_AB && !c->pop[1]) || !c->phi ||
       (need_alt && !c->phi_buf[1]) || !c->mu ||
-      !c->stage || !c->partial || !c->red || !c->step_parts) {
+      !c->stage || !c->partial || !c->red || !c->step_parts ||
+      !c->brick_flags) {
     release(c);
     delete c;
     return fail(nullptr, LBM_ENOMEM, "device allocation failed");
@@ -687,6 +770,7 @@ lbm_status lbm_step(lbm_ctx* c, int n) {
   if (!c) return LBM_EINVAL;
   if (n < 0) return fail(c, LBM_EINVAL, "n must be >= 0");
   if (const lbm_status rs = check_ready(c); rs != LBM_OK) return rs;
+  if (brick_applies(c, n)) return brick_steps(c, n, nullptr);
   int it = 0;
   if (n >= 2 && c->use_graphs && c->vel_kind == LBM_VELOCITY_NONE && !c->profiling &&
       !c->have_prev) {
@@ -722,6 +806,7 @@ lbm_status lbm_step_reduce_async(lbm_ctx* c, int n, double* out_dev) {
     const lbm_status st = lbm_step(c, n);
     return st != LBM_OK ? st : lbm_reduce_async(c, out_dev);
   }
+  if (brick_applies(c, n)) return brick_steps(c, n, out_dev);
   const lbm_status st = lbm_step(c, n - 1);
   return st != LBM_OK ? st : step_once(c, out_dev);
 }
@@ -940,6 +1025,7 @@ lbm_status lbm_set_velocity(lbm_ctx* c, int kind, double U, double period) {
   c->vel_period = kind == LBM_VELOCITY_DEFORMATION ? period : 1.0;
   c->ph.vel_kind = kind;
   c->ph.vel_U = static_cast<float>(U);
+  plan_bricks(c);
   return LBM_OK;
 }
 
@@ -983,6 +1069,10 @@ lbm_status lbm_set_tuning(lbm_ctx* c, int param, int value) {
       if (value > 64) return fail(c, LBM_EINVAL, "LBM_TUNE_FUSED_PREFETCH takes 0..64");
       c->fused_pf = value;
       break;
+    case LBM_TUNE_BRICKS:
+      if (value > 1) return fail(c, LBM_EINVAL, "LBM_TUNE_BRICKS takes 0 or 1");
+      c->use_bricks = value == 1;
+      break;
     default: return fail(c, LBM_EINVAL, "unknown tuning parameter");
   }
   cudaStreamSynchronize(c->stream);  // a replay may still be running
@@ -1009,6 +1099,7 @@ lbm_status lbm_get_tuning(const lbm_ctx* c, int param, int* value) {
     case LBM_TUNE_FUSED: *value = fused_applies(c) ? 1 : 0; return LBM_OK;
     case LBM_TUNE_FUSED_SEGMENT: *value = fused_segment(c); return LBM_OK;
     case LBM_TUNE_FUSED_PREFETCH: *value = c->fused_pf; return LBM_OK;
+    case LBM_TUNE_BRICKS: *value = brick_applies(c, 2) ? 1 : 0; return LBM_OK;
     default: return LBM_EINVAL;
   }
 }
@@ -1057,7 +1148,7 @@ lbm_status lbm_memory_bytes(const lbm_grid* grid, const lbm_params* params, size
   const size_t state = lbm::state_bytes(static_cast<int>(n), params->storage);
   *bytes = state * (params->pattern == LBM_PATTERN_AB ? 2 : 1) +
            plane * (wants_phi_alt(*grid, *params) ? 10 : 9) +
-           sizeof(double) * (5 * lbm::kReduceMaxParts + 8) + step_parts_bytes(n);
+           sizeof(double) * (5 * lbm::kReduceMaxParts + 8) + step_parts_bytes(n) + brick_flag_bytes();
   return LBM_OK;
 }
 

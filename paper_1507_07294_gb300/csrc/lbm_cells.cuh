@@ -287,6 +287,28 @@ __device__ __forceinline__ CellStencils cell_stencils(const float* __restrict__ 
 }
 
 
+// sum_i c_i v_i of a cell's post-collision g (corners (1,1,1), (1,1,-1), (1,-1,1), (1,-1,-1)
+// and their opposites); populations leaving through a wall come back reversed: 2 c_i v_i off.
+__device__ __forceinline__ void momentum_sums(const float v[15], const Nbr& nb, float j[3]) {
+  const float a7 = v[7] - v[8], a9 = v[9] - v[10], a11 = v[11] - v[12], a13 = v[13] - v[14];
+  float jx = (v[1] - v[2]) + ((a7 + a9) + (a11 + a13));
+  float jy = (v[3] - v[4]) + ((a7 + a9) - (a11 + a13));
+  float jz = (v[5] - v[6]) + ((a7 - a9) + (a11 - a13));
+  if (nb.wlo || nb.whi) {
+#define X(I, O, CX, CY, CZ)                                    \
+  if ((CZ > 0 && nb.whi) || (CZ < 0 && nb.wlo)) {              \
+    jx -= 2.0f * CX * v[I];                                    \
+    jy -= 2.0f * CY * v[I];                                    \
+    jz -= 2.0f * CZ * v[I];                                    \
+  }
+    LBM_D3Q15_LIST(X)
+#undef X
+  }
+  j[0] = jx;
+  j[1] = jy;
+  j[2] = jz;
+}
+
 // Pull f and g, stencils of phi and mu, forces, u and p, both MRT collisions,
 // d_t(phi u), store f+ and g+ (Eqs. 14-34).  src and dst are the same array for the
 // in-place patterns.  All 25 cell-state loads are issued first so that they are in
@@ -333,25 +355,7 @@ __device__ __forceinline__ void collide_loaded(float* dst, const Geometry& geo, 
     float v[15];
 #pragma unroll
     for (int i = 0; i < 15; ++i) v[i] = E::get(E::put(g[i]));
-    // sum c_i v_i (corners (1,1,1), (1,1,-1), (1,-1,1), (1,-1,-1) and their opposites)
-    const float a7 = v[7] - v[8], a9 = v[9] - v[10], a11 = v[11] - v[12], a13 = v[13] - v[14];
-    float jx = (v[1] - v[2]) + ((a7 + a9) + (a11 + a13));
-    float jy = (v[3] - v[4]) + ((a7 + a9) - (a11 + a13));
-    float jz = (v[5] - v[6]) + ((a7 - a9) + (a11 - a13));
-    if (nb.wlo || nb.whi) {
-      // populations leaving through a wall come back reversed: take 2 c_i v_i off
-#define X(I, O, CX, CY, CZ)                                    \
-  if ((CZ > 0 && nb.whi) || (CZ < 0 && nb.wlo)) {              \
-    jx -= 2.0f * CX * v[I];                                    \
-    jy -= 2.0f * CY * v[I];                                    \
-    jz -= 2.0f * CZ * v[I];                                    \
-  }
-      LBM_D3Q15_LIST(X)
-#undef X
-    }
-    sums[1] = jx;
-    sums[2] = jy;
-    sums[3] = jz;
+    momentum_sums(v, nb, sums + 1);
   }
   if (P == kAAOdd && use_rows<P>(geo, nb))
     row_store_g_odd<S>(row_pull<S>(dst, nb, idx), g);
@@ -469,23 +473,7 @@ __device__ __forceinline__ void pair_sums(const float2 g[15], const float2 f[7],
   float v[15];
 #pragma unroll
   for (int i = 0; i < 15; ++i) v[i] = E::get(E::put(c ? g[i].y : g[i].x));
-  const float a7 = v[7] - v[8], a9 = v[9] - v[10], a11 = v[11] - v[12], a13 = v[13] - v[14];
-  float jx = (v[1] - v[2]) + ((a7 + a9) + (a11 + a13));
-  float jy = (v[3] - v[4]) + ((a7 + a9) - (a11 + a13));
-  float jz = (v[5] - v[6]) + ((a7 - a9) + (a11 - a13));
-  if (nb.wlo || nb.whi) {
-#define X(I, O_, CX, CY, CZ)                                   \
-  if ((CZ > 0 && nb.whi) || (CZ < 0 && nb.wlo)) {              \
-    jx -= 2.0f * CX * v[I];                                    \
-    jy -= 2.0f * CY * v[I];                                    \
-    jz -= 2.0f * CZ * v[I];                                    \
-  }
-    LBM_D3Q15_LIST(X)
-#undef X
-  }
-  sums[1] = jx;
-  sums[2] = jy;
-  sums[3] = jz;
+  momentum_sums(v, nb, sums + 1);
   float fc[7];
 #pragma unroll
   for (int i = 0; i < 7; ++i) fc[i] = c ? f[i].y : f[i].x;

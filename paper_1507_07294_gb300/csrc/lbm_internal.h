@@ -86,6 +86,47 @@ cudaError_t launch_collide_sums(const float* src, float* dst, const float* phi, 
 cudaError_t launch_step_sums_final(const float* parts, double* partial, double* out,
                                    const Geometry& geo, cudaStream_t st);
 
+// Resident-brick steps of small grids (lbm_brick.cuh): how a grid is cut into bricks, one per
+// block, all resident for a launch of `steps` steps.
+constexpr int kBrickThreads = 256;
+constexpr int kBrickMax = 1024;       // bricks
+constexpr int kBrickFlag = 8;         // ints between two bricks' step counters
+constexpr int kBrickDivShift = 20;
+constexpr int kBrickSteps = 1024;     // most steps of a launch (5-30 ms)
+constexpr int kBrickTrackSteps = 64;  // in tracking mode: one time factor each
+constexpr int kBrickSmem = 200 * 1024;
+enum BrickMode { kBrickCoupled = 0, kBrickTracking = 1 };
+struct BrickPlan {
+  int steps;
+  int nbricks;      // 0: the grid does not go through the kernel
+  int mode, pair;
+  int nb[3], b[3];  // bricks along each axis, cells of the largest along each axis
+  int reach[3];     // bricks along each axis that lie within the cells a step reads
+  int around;       // bricks a block waits for
+  int smem;         // bytes of shared memory
+  unsigned m_qx, m_qy, m_px, m_py, m_mx, m_my, m_bx, m_by;  // small_div of region sizes
+};
+struct BrickTimes {
+  float tf[kBrickTrackSteps];  // time factor of the prescribed velocity at each step of the launch
+};
+// Largest grid whose steps go through the kernel.
+long long brick_most_cells(int mode, int storage);
+// nbricks = 0 where the grid is too large or cannot be cut so that every block is resident.
+BrickPlan brick_plan(const Geometry& geo, const Physics& ph, int mode, int sms);
+// flags: kBrickMax * kBrickFlag step counters, all zero before the first launch; `base` is
+// what every counter holds before this one (each launch adds its steps).  phi: order
+// parameter of the step before (16-bit storage: read, and written by the last of at least two
+// steps).  A block whose wait for its neighbours runs out after `polls` looks sets *err to 1
+// and returns, and so do the others.
+cudaError_t launch_brick(float* state0, float* state1, float* phi, const Geometry& geo,
+                         const Physics& ph, const BrickPlan& plan, const BrickTimes& times, int steps,
+                         int* flags, int base, bool have_prev, int* err, long long polls,
+                         cudaStream_t st);
+// Sums of a state that a step has just written, as launch_collide_sums leaves them in out (5
+// doubles), for grids of up to 2M cells; partial: 5 x kReduceMaxParts doubles, *count zero.
+cudaError_t launch_state_sums(const float* state, const float* phi, const Geometry& geo, double* partial,
+                              double* out, int* count, cudaStream_t st);
+
 // Single-pass step (lbm_fused.cu): pattern AB, default model variant, grids with
 // fused_shape_ok (nx a multiple of 32 with whole-tile rows, ny a multiple of 8).  phi_in
 // and phi_out (distinct arrays) are read and written with 16-bit storage only.  `seg`
