@@ -237,8 +237,9 @@ lbm_status lbm_write_state(lbm_ctx* ctx, const float* f, const float* g,
 /* Tuning parameters (no effect on results, only on speed).
  * LBM_TUNE_PREFETCH_COLLIDE / LBM_TUNE_PREFETCH_PHI: how many thread blocks ahead the
  * fused stream-collide kernel / the order-parameter kernel prefetch cell data into L2
- * (0 disables).  Default: one wave, the number of SMs times the kernel's resident
- * blocks per SM, set by lbm_create.  LBM_TUNE_PREFETCH_COLLIDE_SUMS: the same distance
+ * (0 disables).  Default, set by lbm_create: one wave, the number of SMs times the
+ * kernel's resident blocks per SM; for the FP32 stream-collide kernel a quarter of that
+ * with staged stencils, half without.  LBM_TUNE_PREFETCH_COLLIDE_SUMS: the same distance
  * for the stream-collide kernel of the last step of lbm_step_reduce and
  * lbm_step_reduce_async, which also sums the state it writes and has its own best
  * distance (default: that of LBM_TUNE_PREFETCH_COLLIDE at creation).
@@ -280,7 +281,7 @@ lbm_status lbm_write_state(lbm_ctx* ctx, const float* f, const float* g,
  * LBM_TUNE_STENCIL_STAGE: 1 (default with FP32 populations; 0 with 16-bit ones, where it
  * is slower) lets that two-cell pass (either pattern), on grids whose rows are 64, 128
  * or 256 cells, fetch the rows of phi and mu its block's stencils need into shared
- * memory with TMA bulk copies (one per row and field) instead of loading each stencil
+ * memory with TMA bulk copies (one per plane and field) instead of loading each stencil
  * value per cell; its wait for the copies is bounded like the chemical-potential pass's
  * (LBM_TUNE_TMA_WAIT_POLLS, same error reporting).  lbm_get_tuning reports 1 only while
  * it applies.  Identical results.
@@ -289,10 +290,10 @@ lbm_status lbm_write_state(lbm_ctx* ctx, const float* f, const float* g,
  * interface-tracking mode) by one kernel per call that keeps every block on its own brick of
  * cells for all the steps, blocks waiting for their neighbours between steps.  The wait is
  * bounded; one that runs out is reported as LBM_ETIMEOUT like the TMA passes' waits.
- * lbm_get_tuning reports 1 only while it applies: not while profiling, not while one of the
- * parameters that choose among the three-kernel step's passes (MU_TMA, GRAPHS, ROWS,
- * CELL_PAIRS, STENCIL_STAGE, FUSED, or a poll budget other than the default) is set to
- * anything but its default, and not on a stream under capture.  Identical results.
+ * lbm_get_tuning reports 1 only while it applies: not while profiling or with LBM_TUNE_FUSED,
+ * not on a stream under capture, and not after one of the parameters that choose among the
+ * three-kernel step's passes (MU_TMA, GRAPHS, ROWS, CELL_PAIRS, STENCIL_STAGE,
+ * TMA_WAIT_POLLS) was set, until LBM_TUNE_BRICKS is set again.  Identical results.
  * Setting any parameter drops the captured graphs (and waits for the context's
  * stream).
  * lbm_set_tuning returns LBM_EINVAL for an unknown parameter or a value out of range. */

@@ -53,7 +53,6 @@ struct lbm_ctx {
   long long tma_polls = -1;  // poll budget of the copy's wait; -1: the kernel default
   int row_tiles = 0;         // Geometry::row_tiles when LBM_TUNE_ROWS is on
   int pairs = 0;             // Geometry::pairs when LBM_TUNE_CELL_PAIRS is on
-  int default_stage = 0;     // Geometry::stage as lbm_create set it
   int stage_rows = 0;        // Geometry::stage when LBM_TUNE_STENCIL_STAGE is on
   int prefetch_sums = 0;     // Geometry::prefetch_collide of the steps that sum their result
 
@@ -71,6 +70,7 @@ struct lbm_ctx {
   int brick_base = 0;
   bool brick_reset = true;
   bool use_bricks = true;
+  bool chosen_passes = false;  // the caller set a parameter of the three-kernel step since
 
   // CUDA graphs of two consecutive steps, one per parity of the stored state (which
   // array is current, or the AA step parity, and which phi array is current), replayed
@@ -551,16 +551,13 @@ size_t brick_flag_bytes() {
   return (static_cast<size_t>(lbm::kBrickMax) * lbm::kBrickFlag + 8) * sizeof(int);
 }
 
-// Whether the next n steps go through the resident-brick kernel.  The parameters that
-// choose among the passes of the three-kernel step select that step when set to anything
-// but their defaults, and so does an explicit poll budget (it bounds those passes' copies).
-// A stream under capture takes the three-kernel step too: a replayed launch would find the
-// step counters of its first run.
+// Whether the next n steps go through the resident-brick kernel.  Setting a parameter that
+// chooses among the passes of the three-kernel step, or the poll budget of their copies,
+// selects that step until LBM_TUNE_BRICKS is set again.  A stream under capture takes the
+// three-kernel step too: a replayed launch would find the step counters of its first run.
 bool brick_applies(const lbm_ctx* c, int n) {
-  if (!(c->use_bricks && c->brick.nbricks > 0 && n > 0 && !c->profiling && c->use_graphs &&
-        !fused_applies(c) && c->geo.row_tiles == c->row_tiles && c->geo.pairs == c->pairs &&
-        c->geo.stage == c->default_stage && c->use_phi_map &&
-        (c->tma_polls < 0 || c->tma_polls == lbm::mu_tma_default_polls())))
+  if (!(c->use_bricks && !c->chosen_passes && c->brick.nbricks > 0 && n > 0 && !c->profiling &&
+        !fused_applies(c)))
     return false;
   // with 16-bit storage the first step reads the phi array that the last one writes
   if (n == 1 && c->geo.storage != lbm::kF32) return false;
@@ -665,14 +662,21 @@ lbm_status lbm_create(const lbm_grid* grid, const lbm_params* params, const lbm_
   if (c->pairs && lbm::stage_shape_ok(c->geo)) c->stage_rows = 1;
   // on by default with FP32 populations only: with 16-bit ones the pass is faster
   // loading its stencils per cell (the block waits for all its rows before computing)
-  c->geo.stage = c->default_stage = params->storage == LBM_STORAGE_FP32 ? c->stage_rows : 0;
-  // L2 prefetch distances: one wave of resident blocks
+  c->geo.stage = params->storage == LBM_STORAGE_FP32 ? c->stage_rows : 0;
+  // L2 prefetch distances, in parts of a wave of resident blocks.  The order-parameter pass
+  // and the 16-bit stream-collide, which waits on latency more than on bandwidth, prefetch a
+  // whole wave ahead.  The FP32 stream-collide moves 50 KB a block, and what it prefetches a
+  // wave ahead is partly gone again when it is read: one block per SM ahead is best with
+  // staged stencils (256x256x1024: 1935 us, a wave 2177; 128x128x512: 250, 271), half a wave
+  // without (256x256x256: 493, a wave 509, a quarter 533; 150x141x601: 371, 376, 376).
   {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) == cudaSuccess &&
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess) {
-      c->geo.prefetch_collide =
-          sms * lbm::resident_blocks_per_sm(c->geo.pairs ? 3 : 0, c->geo.storage);
+      const int wave = sms * lbm::resident_blocks_per_sm(c->geo.pairs ? 3 : 0, c->geo.storage);
+      c->geo.prefetch_collide = c->geo.storage != lbm::kF32 ? wave
+                                : c->geo.stage              ? wave / 4
+                                                            : wave / 2;
       c->prefetch_sums = c->geo.prefetch_collide;
       c->geo.prefetch_phi =
           sms * lbm::resident_blocks_per_sm(1, c->geo.storage, c->geo.row_tiles > 0);
@@ -1072,9 +1076,13 @@ lbm_status lbm_set_tuning(lbm_ctx* c, int param, int value) {
     case LBM_TUNE_BRICKS:
       if (value > 1) return fail(c, LBM_EINVAL, "LBM_TUNE_BRICKS takes 0 or 1");
       c->use_bricks = value == 1;
+      c->chosen_passes = false;
       break;
     default: return fail(c, LBM_EINVAL, "unknown tuning parameter");
   }
+  if (param == LBM_TUNE_MU_TMA || param == LBM_TUNE_GRAPHS || param == LBM_TUNE_TMA_WAIT_POLLS ||
+      param == LBM_TUNE_ROWS || param == LBM_TUNE_CELL_PAIRS || param == LBM_TUNE_STENCIL_STAGE)
+    c->chosen_passes = true;
   cudaStreamSynchronize(c->stream);  // a replay may still be running
   drop_graphs(c);                    // their kernel arguments may have changed
   return LBM_OK;

@@ -18,6 +18,8 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "lbm_cells.cuh"
 #include "lbm_device.cuh"
 #include "lbm_internal.h"
@@ -390,19 +392,25 @@ __global__ void __launch_bounds__(kBlock / 2, collide2_min_blocks<S>())
 
 // k_collide2 with the phi and mu stencils staged in shared memory by TMA bulk copies
 // (grids whose rows are 64, 128 or 256 cells: a block's 256 cells are R = 256 / nx whole
-// rows).  For each of its rows and each of the 9 (dy, dz) neighbour rows the stencils
-// use (walls: the ghost of a row beyond the wall is the row itself), thread 0 issues one
-// `cp.async.bulk` of the whole row of phi and one of mu into shared memory (at most 72
-// copies of nx floats, completing on one mbarrier), while every thread loads its two
-// cells' populations; after the (bounded) wait the two x-halo values of each row are
-// filled from the row itself (periodic x) and the cells read their 15-point stencils
-// from shared memory: no stencil load instructions and no stencil registers in flight.
+// rows).  The stencils of those rows reach rows y0 - 1 .. y0 + R of the three planes around
+// them, which lie one after another in memory: the first lanes of warp 0 issue one
+// `cp.async.bulk` for each plane and field (6 in all; a row across the periodic y face by
+// itself; walls: the ghost of a plane beyond the wall is the plane itself), completing on
+// one mbarrier, while every thread loads its two cells' populations.  After the (bounded)
+// wait the cells read their 15-point stencils from shared memory, x neighbours across the
+// periodic face at the other end of the row.  A block whose rows belong to two planes
+// (ny no multiple of R) copies the 9 rows around each of its rows instead.
 // The values are those load_stencil reads, so the state is bit-identical to k_collide2.
-// A block whose wait runs out waits once more (bounded), sets *err as k_mu_tma does,
-// and returns without touching the state.  With SUMS each warp leaves the sums of its
-// two tiles in parts, as k_collide2.
-constexpr int kStRowPad = 8;                            // floats: 4 before, 4 after a row
-constexpr int kStFloats = 9 * 4 * (64 + kStRowPad);    // per field, max over nx = 64..256
+// A warp whose wait runs out waits once more (bounded), sets *err as k_mu_tma does, and
+// returns without touching the state.  With SUMS each warp leaves the sums of its two tiles
+// in parts, as k_collide2.
+// The copies are few and issued by several lanes at once because their issue is on the
+// block's critical path: one thread issuing one copy per row, neighbour row and field (72 a
+// block at nx = 64, 36 at 128, 18 at 256, padded rows and a second barrier to fill their
+// ends) took 53.2 us at 64x64x256, 268 at 128x128x512 and 1939 at 256x256x1024; this way
+// takes 38.5, 250 and 1935, against 37.2, 249 and 1961 of k_collide2 at its best prefetch
+// distance.
+constexpr int kStFloats = 9 * 256;  // per field: 3 planes of (R + 2) nx floats, or 9 R rows
 
 __device__ __forceinline__ void bulk_row(unsigned dst, const float* src, unsigned bytes,
                                          unsigned bar) {
@@ -410,6 +418,29 @@ __device__ __forceinline__ void bulk_row(unsigned dst, const float* src, unsigne
       "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
       "l"(src), "r"(bytes), "r"(bar)
       : "memory");
+}
+
+// The stencils of cells x and x + kTile of a staged row: c points at its column 0, rows lie
+// NX floats apart and planes SZ (compile-time, so that every load is a base and a constant).
+template <int NX, int SZ>
+__device__ __forceinline__ StencilV<float2> staged_stencil(const float* c, int x, const Nbr& na,
+                                                           const Nbr& nb2) {
+  const float *c0 = c + x, *m0 = c0 + na.xm, *p0 = c0 + na.xp;
+  const float *c1 = c0 + kTile, *m1 = c1 + nb2.xm, *p1 = c1 + nb2.xp;
+  StencilV<float2> s;
+  s.c = make_float2(c0[0], c1[0]);
+  s.xm = make_float2(m0[0], m1[0]);
+  s.xp = make_float2(p0[0], p1[0]);
+  s.ym = make_float2(c0[-NX], c1[-NX]);
+  s.yp = make_float2(c0[NX], c1[NX]);
+  s.zm = make_float2(c0[-SZ], c1[-SZ]);
+  s.zp = make_float2(c0[SZ], c1[SZ]);
+#pragma unroll
+  for (int b = 0; b < 8; ++b) {
+    const int o = ((b & 2) ? NX : -NX) + ((b & 4) ? SZ : -SZ);
+    s.k[b] = (b & 1) ? make_float2(p0[o], p1[o]) : make_float2(m0[o], m1[o]);
+  }
+  return s;
 }
 
 template <int VAR, int S, bool SUMS, int P = kAB>
@@ -421,31 +452,48 @@ __global__ void __launch_bounds__(kBlock / 2, collide2_min_blocks<S>())
   __shared__ alignas(8) unsigned long long bar_storage;
   prefetch_ahead<S, true>(src, phi, mu, geo, geo.prefetch_collide);
   const unsigned bar = smem_addr(&bar_storage);
-  const int nx = geo.nx, R = kBlock / nx, stride = nx + kStRowPad;
+  const int nx = geo.nx, R = kBlock / nx;
   const int b0 = blockIdx.x * kBlock;
   const int rows = min(R, (geo.n - b0) / nx);  // whole rows of this block
-  if (threadIdx.x == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  const int row0 = fast_div(b0, geo.div_nx);   // its first row: y0 + ny z0
+  const int z0 = fast_div(row0, geo.div_ny), y0 = row0 - z0 * geo.ny;
+  const bool split = y0 + rows > geo.ny;       // the rows belong to several planes
+  if (threadIdx.x < 32) {
     const unsigned row_bytes = static_cast<unsigned>(nx) * 4u;
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
-                 "r"(2u * 9u * static_cast<unsigned>(rows) * row_bytes)
-                 : "memory");
-    for (int r = 0; r < rows; ++r) {
-      const int gr = b0 / nx + r;  // global row index: y + ny z
-      const int z = gr / geo.ny, y = gr - z * geo.ny;
-      for (int k = 0; k < 9; ++k) {
-        const int dy = k % 3 - 1, dz = k / 3 - 1;
+    if (threadIdx.x == 0) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
+                   "r"((split ? 18u * rows : 6u * (rows + 2)) * row_bytes)
+                   : "memory");
+    }
+    __syncwarp();
+    auto plane_z = [&](int z, int dz) {
+      const int zz = z + dz;
+      if (geo.walls) return (zz < 0 || zz >= geo.nz) ? z : zz;
+      return zz < 0 ? geo.nz - 1 : (zz >= geo.nz ? 0 : zz);
+    };
+    if (!split) {
+      // lane: piece 0 the row below across the periodic face (y0 = 0), 1 the rows that
+      // follow one another, 2 the row above across the face (y0 + rows = ny)
+      const int piece = threadIdx.x / 6, q = threadIdx.x - 6 * piece, field = q / 3, dz = q - 3 * field;
+      const bool lo = y0 == 0, hi = y0 + rows == geo.ny;
+      if (piece < 3 && (piece == 1 || (piece == 0 ? lo : hi))) {
+        const int first = piece == 1 ? y0 - (lo ? 0 : 1) : (piece == 0 ? geo.ny - 1 : 0);
+        const int count = piece == 1 ? rows + (lo ? 0 : 1) + (hi ? 0 : 1) : 1;
+        const int at = piece == 1 ? (lo ? 1 : 0) : (piece == 0 ? 0 : rows + 1);
+        const size_t from = (static_cast<size_t>(plane_z(z0, dz - 1)) * geo.ny + first) * nx;
+        bulk_row(smem_addr(&st[field][(dz * (R + 2) + at) * nx]), (field ? mu : phi) + from,
+                 count * row_bytes, bar);
+      }
+    } else {
+      for (int k = threadIdx.x; k < 18 * rows; k += 32) {
+        const int field = k / (9 * rows), q = k - field * 9 * rows, r = q / 9, j = q - 9 * r;
+        const int dz = j / 3 - 1, dy = j - 3 * (j / 3) - 1;
+        const int z = fast_div(row0 + r, geo.div_ny), y = row0 + r - z * geo.ny;
         const int yy = y + dy < 0 ? geo.ny - 1 : (y + dy >= geo.ny ? 0 : y + dy);
-        int zz = z + dz;
-        if (geo.walls)
-          zz = (zz < 0 || zz >= geo.nz) ? z : zz;
-        else
-          zz = zz < 0 ? geo.nz - 1 : (zz >= geo.nz ? 0 : zz);
-        const size_t row0 = (static_cast<size_t>(zz) * geo.ny + yy) * nx;
-        const int off = (r * 9 + k) * stride + 4;
-        bulk_row(smem_addr(&st[0][off]), phi + row0, row_bytes, bar);
-        bulk_row(smem_addr(&st[1][off]), mu + row0, row_bytes, bar);
+        const size_t from = (static_cast<size_t>(plane_z(z, dz)) * geo.ny + yy) * nx;
+        bulk_row(smem_addr(&st[field][(r * 9 + j) * nx]), (field ? mu : phi) + from, row_bytes, bar);
       }
     }
   }
@@ -461,67 +509,33 @@ __global__ void __launch_bounds__(kBlock / 2, collide2_min_blocks<S>())
     load_cell<P, S, true>(src, geo, idx + kTile, nb2, gb, fb, pb);
   }
   __syncthreads();  // the barrier is initialised and armed before anyone polls it
-  if (!__syncthreads_and(mbar_wait(bar, 0, polls))) {
-    if (threadIdx.x == 0) atomicMax(err, mbar_wait(bar, 0, kMbarSpins) ? 1 : 2);
-    __syncthreads();
+  if (!__all_sync(0xffffffffu, mbar_wait(bar, 0, polls))) {
+    const bool landed = mbar_wait(bar, 0, kMbarSpins);
+    if ((threadIdx.x & 31) == 0) atomicMax(err, landed ? 1 : 2);
     return;
   }
-  // periodic x halo of every row copy: column -1 = nx - 1, column nx = 0
-  for (int k = threadIdx.x; k < 2 * 9 * rows * 2; k += blockDim.x) {
-    const int side = k & 1, rk = (k >> 1) % (9 * rows), f = (k >> 1) / (9 * rows);
-    float* row = &st[f][rk * stride + 4];
-    if (side)
-      row[nx] = row[0];
-    else
-      row[-1] = row[nx - 1];
-  }
-  __syncthreads();
   // with SUMS every lane of a warp takes part in the warp sums; a warp is wholly inside
   // or outside the grid (n is a multiple of 64)
   if (!active) return;
-  // stencil of the cell at x in block row r from the staged rows (k = 3 (dz + 1) + dy + 1)
-  const int r = (idx - b0) / nx;
-  auto stencil = [&](const float* a, int xc) {
-    const float* base = a + r * 9 * stride + 4 + xc;
-    auto row = [&](int dy, int dz) { return base + (3 * (dz + 1) + dy + 1) * stride; };
-    Stencil s;
-    s.c = row(0, 0)[0];
-    s.xm = row(0, 0)[-1];
-    s.xp = row(0, 0)[1];
-    s.ym = row(-1, 0)[0];
-    s.yp = row(1, 0)[0];
-    s.zm = row(0, -1)[0];
-    s.zp = row(0, 1)[0];
-#pragma unroll
-    for (int b = 0; b < 8; ++b)
-      s.k[b] = row((b & 2) ? 1 : -1, (b & 4) ? 1 : -1)[(b & 1) ? 1 : -1];
-    return s;
-  };
   StencilV<float2> sp, sm;
-  {
-    const Stencil s0 = stencil(st[0], x), s1 = stencil(st[0], x + kTile);
-    sp.c = make_float2(s0.c, s1.c);
-    sp.xm = make_float2(s0.xm, s1.xm);
-    sp.xp = make_float2(s0.xp, s1.xp);
-    sp.ym = make_float2(s0.ym, s1.ym);
-    sp.yp = make_float2(s0.yp, s1.yp);
-    sp.zm = make_float2(s0.zm, s1.zm);
-    sp.zp = make_float2(s0.zp, s1.zp);
-#pragma unroll
-    for (int b = 0; b < 8; ++b) sp.k[b] = make_float2(s0.k[b], s1.k[b]);
-  }
-  {
-    const Stencil s0 = stencil(st[1], x), s1 = stencil(st[1], x + kTile);
-    sm.c = make_float2(s0.c, s1.c);
-    sm.xm = make_float2(s0.xm, s1.xm);
-    sm.xp = make_float2(s0.xp, s1.xp);
-    sm.ym = make_float2(s0.ym, s1.ym);
-    sm.yp = make_float2(s0.yp, s1.yp);
-    sm.zm = make_float2(s0.zm, s1.zm);
-    sm.zp = make_float2(s0.zp, s1.zp);
-#pragma unroll
-    for (int b = 0; b < 8; ++b) sm.k[b] = make_float2(s0.k[b], s1.k[b]);
-  }
+  const int r = (idx - b0) / nx;  // the cell's row in the block
+  auto read = [&](auto nxc, auto szc) {
+    constexpr int NX = decltype(nxc)::value, SZ = decltype(szc)::value;
+    const int c = (SZ == 3 * NX && split ? 9 * r + 4 : SZ / NX + r + 1) * NX;
+    sp = staged_stencil<NX, SZ>(&st[0][c], x, na, nb2);
+    sm = staged_stencil<NX, SZ>(&st[1][c], x, na, nb2);
+  };
+  typedef std::integral_constant<int, 64> I64;
+  typedef std::integral_constant<int, 128> I128;
+  typedef std::integral_constant<int, 256> I256;
+  if (nx == 256)
+    read(I256{}, std::integral_constant<int, 3 * 256>{});
+  else if (nx == 128)
+    split ? read(I128{}, std::integral_constant<int, 3 * 128>{})
+          : read(I128{}, std::integral_constant<int, 4 * 128>{});
+  else
+    split ? read(I64{}, std::integral_constant<int, 3 * 64>{})
+          : read(I64{}, std::integral_constant<int, 6 * 64>{});
   float2 g[15], f[7], prev[3], cur[3];
 #pragma unroll
   for (int i = 0; i < 15; ++i) g[i] = make_float2(ga[i], gb[i]);
