@@ -62,11 +62,9 @@ STEP_BYTES_PER_CELL = COLLIDE_BYTES_PER_CELL + (7 + 1) * 4 + (1 + 1) * 4  # + k_
 COLLIDE_BYTES_PER_CELL_16 = 2 * (22 * 2 + 12) + 8
 STEP_BYTES_PER_CELL_16 = COLLIDE_BYTES_PER_CELL_16 + (7 * 2 + 4 + 4) + 8
 
-# Interface tracking with a prescribed velocity (k_che): read f, phi and mu at the cell
-# and phi u of the previous step (48 B), write f and phi u (40 B); the step adds k_phi
-# and k_mu.
-CHE_BYTES_PER_CELL = (7 + 1 + 1 + 3) * 4 + (7 + 3) * 4
-CHE_STEP_BYTES_PER_CELL = CHE_BYTES_PER_CELL + (7 + 1) * 4 + (1 + 1) * 4
+# Interface tracking with a prescribed velocity: one kernel (k_track_rows) reads f and phi u
+# of the previous step (40 B) and writes both (40 B).
+TRACK_BYTES_PER_CELL = 2 * (7 + 3) * 4
 
 # The one-kernel step (k_fused): the state read and written once (200 B in FP32); with
 # 16-bit populations 2 x (44 + 12) plus phi of the previous step read and the new phi
@@ -618,8 +616,8 @@ def run_ours(args):
             mruns = [("srt_flow", srt, "k_collide", COLLIDE_BYTES_PER_CELL, STEP_BYTES_PER_CELL),
                      ("d3q7_stencil", d7, "k_collide", COLLIDE_BYTES_PER_CELL,
                       STEP_BYTES_PER_CELL),
-                     ("interface_tracking", I.deformation(n=256), "k_che", CHE_BYTES_PER_CELL,
-                      CHE_STEP_BYTES_PER_CELL)]
+                     ("interface_tracking", I.deformation(n=256), "k_track_rows",
+                      TRACK_BYTES_PER_CELL, TRACK_BYTES_PER_CELL)]
             for name, wv, kname, cb, sb in mruns:
                 vs = L.Solver(wv, stream=stream.cuda_stream)
                 vs.step(args.warmup)

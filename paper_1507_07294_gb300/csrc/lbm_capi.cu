@@ -456,6 +456,17 @@ lbm_status step_once(lbm_ctx* c, double* sums_out) {
     ++c->step;
     return LBM_OK;
   }
+  if (c->vel_kind != LBM_VELOCITY_NONE && c->params.pattern == LBM_PATTERN_AB &&
+      lbm::track_shape_ok(c->geo)) {
+    const float tf = velocity_time_factor(c, c->step);
+    LBM_CK(c, timed(c, 2, [&] {
+             return lbm::launch_track(src, dst, c->geo, c->ph, c->have_prev, tf, c->stream);
+           }));
+    c->cur = 1 - c->cur;
+    c->have_prev = true;
+    ++c->step;
+    return LBM_OK;
+  }
   LBM_CK(c, timed(c, 0, [&] { return lbm::launch_phi(src, c->phi, c->phi, c->geo, pat, c->stream); }));
   LBM_CK(c, timed(c, 1, [&] {
            return c->have_phi_map && c->use_phi_map

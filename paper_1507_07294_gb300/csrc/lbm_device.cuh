@@ -488,6 +488,14 @@ __device__ __forceinline__ void load_stencil(const float* __restrict__ a, int id
 //   uniform:     (U, 0, 0)
 //   rotation:    Eq. 37, v = -Omega (z - N/2), w = Omega (y - N/2), Omega = U pi / N, N = ny
 //   deformation: Eq. 41 with L = nx.
+// The deformation field from sin(pi x / L) and sin(2 pi x / L) of the three axes.
+__device__ __forceinline__ void deformation_velocity(float U, float tf, float sx, float s2x, float sy,
+                                                     float s2y, float sz, float s2z, float u[3]) {
+  u[0] = 2.0f * U * sx * sx * s2y * s2z * tf;
+  u[1] = -U * s2x * sy * sy * s2z * tf;
+  u[2] = -U * s2x * s2y * sz * sz * tf;
+}
+
 __device__ __forceinline__ void prescribed_velocity(const Physics& ph, const Geometry& geo, int x,
                                                     int y, int z, float tf, float u[3]) {
   const float U = ph.vel_U;
@@ -505,11 +513,8 @@ __device__ __forceinline__ void prescribed_velocity(const Physics& ph, const Geo
     const float inv_l = 1.0f / static_cast<float>(geo.nx);
     const float ax = static_cast<float>(x) * inv_l, ay = static_cast<float>(y) * inv_l,
                 az = static_cast<float>(z) * inv_l;
-    const float sx = sinpif(ax), sy = sinpif(ay), sz = sinpif(az);
-    const float s2x = sinpif(2.0f * ax), s2y = sinpif(2.0f * ay), s2z = sinpif(2.0f * az);
-    u[0] = 2.0f * U * sx * sx * s2y * s2z * tf;
-    u[1] = -U * s2x * sy * sy * s2z * tf;
-    u[2] = -U * s2x * s2y * sz * sz * tf;
+    deformation_velocity(U, tf, sinpif(ax), sinpif(2.0f * ax), sinpif(ay), sinpif(2.0f * ay),
+                         sinpif(az), sinpif(2.0f * az), u);
   }
 }
 

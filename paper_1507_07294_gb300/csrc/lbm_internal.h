@@ -43,6 +43,11 @@ bool stage_shape_ok(const Geometry& geo);
 cudaError_t launch_che(const float* src, float* dst, const float* phi, const float* mu,
                        const Geometry& geo, const Physics& ph, int pattern, bool have_prev,
                        float tf, cudaStream_t st);
+// One-pass tracking step (lbm_track.cu): phi, mu and launch_che's collision in one kernel,
+// pattern AB, for grids with track_shape_ok.
+bool track_shape_ok(const Geometry& geo);
+cudaError_t launch_track(const float* src, float* dst, const Geometry& geo, const Physics& ph,
+                         bool have_prev, float tf, cudaStream_t st);
 cudaError_t launch_fields(const float* src, const float* phi, const float* mu, float* out,
                           const Geometry& geo, const Physics& ph, int pattern, float tf,
                           cudaStream_t st);
