@@ -7,13 +7,13 @@ namespace lbm {
 
 const void* brick_kernel_f32(int mode, int var, bool pair);
 cudaError_t state_sums_f32(const float* state, const float* phi, const Geometry& geo, double* partial,
-                        double* out, int* count, cudaStream_t st);
+                        double* out, const double* word, int* count, cudaStream_t st);
 const void* brick_kernel_f16(int mode, int var, bool pair);
 cudaError_t state_sums_f16(const float* state, const float* phi, const Geometry& geo, double* partial,
-                        double* out, int* count, cudaStream_t st);
+                        double* out, const double* word, int* count, cudaStream_t st);
 const void* brick_kernel_bf16(int mode, int var, bool pair);
 cudaError_t state_sums_bf16(const float* state, const float* phi, const Geometry& geo, double* partial,
-                        double* out, int* count, cudaStream_t st);
+                        double* out, const double* word, int* count, cudaStream_t st);
 
 namespace {
 
@@ -170,15 +170,18 @@ cudaError_t launch_brick(float* state0, float* state1, float* phi, const Geometr
   int hp = have_prev ? 1 : 0;
   void* args[] = {&state0, &state1, &phi, const_cast<Geometry*>(&geo), const_cast<Physics*>(&ph), &bp,
                   const_cast<BrickTimes*>(&times), &flags, &base, &hp, &err, &polls};
-  return cudaLaunchCooperativeKernel(kernel_of(geo, ph, plan.mode, plan.pair != 0), dim3(plan.nbricks),
-                                     dim3(kBrickThreads), args, plan.smem, st);
+  const void* k = kernel_of(geo, ph, plan.mode, plan.pair != 0);
+  // in a single step no block waits for another, so they need not be resident together
+  return steps == 1
+             ? cudaLaunchKernel(k, dim3(plan.nbricks), dim3(kBrickThreads), args, plan.smem, st)
+             : cudaLaunchCooperativeKernel(k, dim3(plan.nbricks), dim3(kBrickThreads), args, plan.smem, st);
 }
 
 cudaError_t launch_state_sums(const float* state, const float* phi, const Geometry& geo, double* partial,
-                              double* out, int* count, cudaStream_t st) {
-  return geo.storage == kF16    ? state_sums_f16(state, phi, geo, partial, out, count, st)
-         : geo.storage == kBF16 ? state_sums_bf16(state, phi, geo, partial, out, count, st)
-                                : state_sums_f32(state, phi, geo, partial, out, count, st);
+                              double* out, const double* word, int* count, cudaStream_t st) {
+  return geo.storage == kF16    ? state_sums_f16(state, phi, geo, partial, out, word, count, st)
+         : geo.storage == kBF16 ? state_sums_bf16(state, phi, geo, partial, out, word, count, st)
+                                : state_sums_f32(state, phi, geo, partial, out, word, count, st);
 }
 
 }  // namespace lbm

@@ -406,7 +406,7 @@ __global__ void __launch_bounds__(kBlock) k_state_sums(const float* __restrict__
                                                        const __grid_constant__ Geometry geo,
                                                        int ntiles, int chunk,
                                                        double* __restrict__ partial, double* out,
-                                                       int* count) {
+                                                       const double* word, int* count) {
   __shared__ float parts[kSumTiles * 5];
   __shared__ int s_last;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -465,17 +465,20 @@ __global__ void __launch_bounds__(kBlock) k_state_sums(const float* __restrict__
     for (int o = 16; o > 0; o >>= 1) r += __shfl_down_sync(0xffffffffu, r, o);
     if (lane == 0) out[warp] = r;
   }
-  if (threadIdx.x == 0) *count = 0;
+  if (threadIdx.x == 0) {
+    *count = 0;
+    if (word) out[7] = *word;
+  }
 }
 
 template <int S>
 cudaError_t state_sums(const float* state, const float* phi, const Geometry& geo, double* partial,
-                       double* out, int* count, cudaStream_t st) {
+                       double* out, const double* word, int* count, cudaStream_t st) {
   const int ntiles = cell_warps(geo.n);
   const int groups = ntiles < kReduceMaxParts ? ntiles : kReduceMaxParts;
   const int chunk = (ntiles + groups - 1) / groups;
   if (chunk > kSumTiles) return cudaErrorInvalidValue;
-  k_state_sums<S><<<groups, kBlock, 0, st>>>(state, phi, geo, ntiles, chunk, partial, out, count);
+  k_state_sums<S><<<groups, kBlock, 0, st>>>(state, phi, geo, ntiles, chunk, partial, out, word, count);
   return cudaGetLastError();
 }
 

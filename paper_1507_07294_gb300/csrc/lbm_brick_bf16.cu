@@ -6,8 +6,8 @@ namespace lbm {
 const void* brick_kernel_bf16(int mode, int var, bool pair) { return brick_kernel<kBF16>(mode, var, pair); }
 
 cudaError_t state_sums_bf16(const float* state, const float* phi, const Geometry& geo, double* partial,
-                           double* out, int* count, cudaStream_t st) {
-  return state_sums<kBF16>(state, phi, geo, partial, out, count, st);
+                           double* out, const double* word, int* count, cudaStream_t st) {
+  return state_sums<kBF16>(state, phi, geo, partial, out, word, count, st);
 }
 
 }  // namespace lbm

@@ -42,6 +42,9 @@ struct lbm_ctx {
                            // gather/scatter, initial u and p
   double* partial = nullptr;  // reduction partials
   double* red = nullptr;      // 5 reduction results; red[7] holds the device error word
+  double* host_red = own_red;  // where the host reads them: a page-locked slot where there is one
+  double* slot_dev = nullptr;  // that slot's device address
+  double own_red[8] = {};
   float* step_parts = nullptr;   // per-warp partials of the fused step sums (FP32 sums of
                                  // 32 cells and a count: exact in float)
 
@@ -131,6 +134,42 @@ void dev_free(lbm_ctx* c, void* p) {
     c->alloc.free(p, c->alloc.user);
   else
     cudaFree(p);
+}
+
+// Page-locked slots of 8 doubles for the results that the host waits for: the last kernel of a
+// reduction stores them there itself, where a copy into pageable memory would be one more
+// enqueued operation and pass through the driver's staging (32^3, lbm_step_reduce of one step: 41 ->
+// 37 us a call, lbm_reduce 32 -> 28).  One page, mapped by the first context that asks and kept; contexts beyond its
+// 64 slots, or where it cannot be had, copy into their own memory.
+struct RedSlots {
+  std::mutex lock;
+  double* page = nullptr;
+  bool tried = false;
+  unsigned long long used = 0;
+};
+RedSlots g_red_slots;
+
+double* take_red_slot() {
+  std::lock_guard<std::mutex> hold(g_red_slots.lock);
+  RedSlots& r = g_red_slots;
+  if (!r.tried) {
+    r.tried = true;
+    void* p = nullptr;
+    if (cudaHostAlloc(&p, 64 * 8 * sizeof(double), cudaHostAllocPortable | cudaHostAllocMapped) == cudaSuccess)
+      r.page = static_cast<double*>(p);
+    else
+      cudaGetLastError();
+  }
+  if (!r.page || r.used == ~0ull) return nullptr;
+  int k = 0;
+  while (r.used >> k & 1) ++k;
+  r.used |= 1ull << k;
+  return r.page + 8 * k;
+}
+
+void give_red_slot(double* slot) {
+  std::lock_guard<std::mutex> hold(g_red_slots.lock);
+  g_red_slots.used &= ~(1ull << ((slot - g_red_slots.page) / 8));
 }
 
 bool rate_ok(double s) { return s > 0.0 && s < 2.0 && std::isfinite(s); }
@@ -229,6 +268,9 @@ void release(lbm_ctx* c) {
   dev_free(c, c->red);
   dev_free(c, c->step_parts);
   dev_free(c, c->brick_flags);
+  if (c->slot_dev) give_red_slot(c->host_red);
+  c->host_red = c->own_red;
+  c->slot_dev = nullptr;
   c->pop[0] = c->pop[1] = c->phi = c->phi_buf[0] = c->phi_buf[1] = c->mu = c->stage = nullptr;
   c->partial = c->red = nullptr;
   c->step_parts = nullptr;
@@ -435,7 +477,7 @@ namespace {
 
 // One time step; with sums_out the stream-collide pass also reduces the new state into
 // sums_out (5 doubles on the device; coupled default variant only).
-lbm_status step_once(lbm_ctx* c, double* sums_out) {
+lbm_status step_once(lbm_ctx* c, double* sums_out, const double* word = nullptr) {
   const int pat = read_pattern(c);
   const float* src = cur_state(c);
   float* dst = c->params.pattern == LBM_PATTERN_AB ? c->pop[1 - c->cur] : c->pop[c->cur];
@@ -445,7 +487,7 @@ lbm_status step_once(lbm_ctx* c, double* sums_out) {
              return lbm::launch_fused(src, dst, c->phi, phi_out, c->geo, c->ph, c->have_prev,
                                       fused_segment(c), c->fused_pf,
                                       sums_out ? c->step_parts : nullptr, c->partial, sums_out,
-                                      c->stream);
+                                      c->stream, word);
            }));
     if (phi_out) {
       c->phi_sel = 1 - c->phi_sel;
@@ -487,7 +529,8 @@ lbm_status step_once(lbm_ctx* c, double* sums_out) {
                                                          sums_out, c->stream, error_word(c),
                                                          c->tma_polls < 0
                                                              ? lbm::mu_tma_default_polls()
-                                                             : c->tma_polls)
+                                                             : c->tma_polls,
+                                                         word)
                              : lbm::launch_collide(src, dst, c->phi, c->mu, c->geo, c->ph, pat,
                                                    prev, c->stream, error_word(c),
                                                    c->tma_polls < 0 ? lbm::mu_tma_default_polls()
@@ -558,6 +601,8 @@ lbm_status capture_pair(lbm_ctx* c, int parity) {
   return LBM_OK;
 }
 
+lbm_status step_sums(lbm_ctx* c, int n, double* out, const double* word);
+
 size_t brick_flag_bytes() {
   return (static_cast<size_t>(lbm::kBrickMax) * lbm::kBrickFlag + 8) * sizeof(int);
 }
@@ -577,7 +622,7 @@ bool brick_applies(const lbm_ctx* c, int n) {
 }
 
 // n steps through the resident-brick kernel; with sums_out the sums of the state after them.
-lbm_status brick_steps(lbm_ctx* c, int n, double* sums_out) {
+lbm_status brick_steps(lbm_ctx* c, int n, double* sums_out, const double* word = nullptr) {
   const bool tracking = c->vel_kind != LBM_VELOCITY_NONE;
   while (n > 0) {
     const int most = tracking ? lbm::kBrickTrackSteps : lbm::kBrickSteps;
@@ -599,7 +644,7 @@ lbm_status brick_steps(lbm_ctx* c, int n, double* sums_out) {
       // fewer SMs than the device has (a partition of it): the three-kernel step from here on
       cudaGetLastError();
       c->brick = lbm::BrickPlan{};
-      return sums_out ? lbm_step_reduce_async(c, n, sums_out) : lbm_step(c, n);
+      return sums_out ? step_sums(c, n, sums_out, word) : lbm_step(c, n);
     }
     LBM_CK(c, e);
     c->brick_base += k;
@@ -609,7 +654,7 @@ lbm_status brick_steps(lbm_ctx* c, int n, double* sums_out) {
     n -= k;
   }
   if (sums_out)
-    LBM_CK(c, lbm::launch_state_sums(c->pop[c->cur], c->phi, c->geo, c->partial, sums_out,
+    LBM_CK(c, lbm::launch_state_sums(c->pop[c->cur], c->phi, c->geo, c->partial, sums_out, word,
                                      c->brick_flags + lbm::kBrickMax * lbm::kBrickFlag, c->stream));
   return LBM_OK;
 }
@@ -627,6 +672,37 @@ void plan_bricks(lbm_ctx* c) {
 bool fused_sums(const lbm_ctx* c) {
   return c->vel_kind == LBM_VELOCITY_NONE &&
          !(c->params.flags & (LBM_FLAG_SRT_FLOW | LBM_FLAG_D3Q7_STENCIL));
+}
+
+// Where the reductions whose result the host waits for put it: straight into the page-locked
+// slot, with the error word, or into red, which fetch_results then copies.
+double* result_target(lbm_ctx* c) { return c->slot_dev ? c->slot_dev : c->red; }
+const double* result_word(const lbm_ctx* c) { return c->slot_dev ? c->red + 7 : nullptr; }
+
+// Waits for the context's stream; the results and the error word are then in host_red.
+cudaError_t fetch_results(lbm_ctx* c) {
+  if (!c->slot_dev) {
+    const cudaError_t e = cudaMemcpyAsync(c->host_red, c->red, 8 * sizeof(double),
+                                          cudaMemcpyDeviceToHost, c->stream);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaStreamSynchronize(c->stream);
+}
+
+// n steps and the sums of the state after them in out[0..4] (and `word` in out[7]).
+lbm_status step_sums(lbm_ctx* c, int n, double* out, const double* word) {
+  if (!fused_sums(c)) {
+    const lbm_status st = lbm_step(c, n);
+    if (st != LBM_OK) return st;
+    float* phi_now = c->stage + 5 * c->geo.stride;
+    LBM_CK(c, lbm::launch_phi(cur_state(c), c->phi, phi_now, c->geo, read_pattern(c), c->stream));
+    LBM_CK(c, lbm::launch_reduce(cur_state(c), phi_now, c->partial, out, c->geo, read_pattern(c),
+                                 c->vel_kind == LBM_VELOCITY_NONE, c->stream, word));
+    return LBM_OK;
+  }
+  if (brick_applies(c, n)) return brick_steps(c, n, out, word);
+  const lbm_status st = lbm_step(c, n - 1);
+  return st != LBM_OK ? st : step_once(c, out, word);
 }
 
 }  // namespace
@@ -733,6 +809,13 @@ lbm_status lbm_create(const lbm_grid* grid, const lbm_params* params, const lbm_
     delete c;
     return fail(nullptr, LBM_ECUDA, std::string("cudaMemsetAsync: ") + cudaGetErrorString(e));
   }
+  if (double* slot = take_red_slot()) {
+    c->slot_dev = device_view(slot);
+    if (c->slot_dev)
+      c->host_red = slot;
+    else
+      give_red_slot(slot);
+  }
   *out = c;
   return LBM_OK;
 }
@@ -817,23 +900,18 @@ lbm_status lbm_step_reduce_async(lbm_ctx* c, int n, double* out_dev) {
   if (!out_dev || reinterpret_cast<uintptr_t>(out_dev) % alignof(double) != 0)
     return fail(c, LBM_EINVAL, "out_dev must be a non-NULL, 8-byte aligned pointer");
   if (const lbm_status rs = check_ready(c); rs != LBM_OK) return rs;
-  if (!fused_sums(c)) {
-    const lbm_status st = lbm_step(c, n);
-    return st != LBM_OK ? st : lbm_reduce_async(c, out_dev);
-  }
-  if (brick_applies(c, n)) return brick_steps(c, n, out_dev);
-  const lbm_status st = lbm_step(c, n - 1);
-  return st != LBM_OK ? st : step_once(c, out_dev);
+  return step_sums(c, n, out_dev, nullptr);
 }
 
 lbm_status lbm_step_reduce(lbm_ctx* c, int n, double* sum_phi, double mom[3]) {
   if (!c) return LBM_EINVAL;
   if (!sum_phi || !mom) return fail(c, LBM_EINVAL, "outputs must not be NULL");
-  const lbm_status st = lbm_step_reduce_async(c, n, c->red);
+  if (n < 1) return fail(c, LBM_EINVAL, "n must be >= 1");
+  if (const lbm_status rs = check_ready(c); rs != LBM_OK) return rs;
+  const lbm_status st = step_sums(c, n, result_target(c), result_word(c));
   if (st != LBM_OK) return st;
-  double h[8];
-  LBM_CK(c, cudaMemcpyAsync(h, c->red, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
-  LBM_CK(c, cudaStreamSynchronize(c->stream));
+  const double* h = c->host_red;
+  LBM_CK(c, fetch_results(c));
   if (const lbm_status te = take_device_error(c, h); te != LBM_OK) return te;
   *sum_phi = h[0];
   mom[0] = h[1];
@@ -851,42 +929,59 @@ lbm_status lbm_read_fields(lbm_ctx* c, unsigned mask, double* phi, double* rho, 
   if (((mask & LBM_FIELD_PHI) && !phi) || ((mask & LBM_FIELD_RHO) && !rho) ||
       ((mask & LBM_FIELD_P) && !p) || ((mask & LBM_FIELD_U) && !u) || ((mask & LBM_FIELD_MU) && !mu))
     return fail(c, LBM_EINVAL, "a selected field has a NULL buffer");
-  // phi and mu of the current state into staging planes 5 and 6: the solver's own phi
-  // array is the reference of the 16-bit slot 0 and must keep the previous step's phi.
   const size_t n = static_cast<size_t>(c->geo.n);
   const size_t s = c->geo.stride;
+  const unsigned flow = LBM_FIELD_RHO | LBM_FIELD_P | LBM_FIELD_U;
+  const float tf = velocity_time_factor(c, c->step);
+  bool pageable = false;
+  auto view = [&](unsigned bit, double* host) -> double* {
+    if (!(mask & bit)) return nullptr;
+    double* v = device_view(host);
+    pageable = pageable || !v;
+    return v;
+  };
+  double *vphi = view(LBM_FIELD_PHI, phi), *vrho = view(LBM_FIELD_RHO, rho), *vp = view(LBM_FIELD_P, p),
+         *vu = view(LBM_FIELD_U, u), *vmu = view(LBM_FIELD_MU, mu);
+  // u is written through one address: its three planes have to be one mapping
+  if (vu && (device_view(u + n) != vu + n || device_view(u + 2 * n) != vu + 2 * n)) pageable = true;
+  // phi and mu of the current state into staging planes 5 and 6: the solver's own phi
+  // array is the reference of the 16-bit slot 0 and must keep the previous step's phi.
   float* phi_now = c->stage + 5 * s;
   float* mu_now = c->stage + 6 * s;
-  LBM_CK(c, lbm::launch_phi(cur_state(c), c->phi, phi_now, c->geo, read_pattern(c), c->stream));
-  LBM_CK(c, lbm::launch_mu(phi_now, mu_now, c->geo, c->ph, c->stream));
-  if (mask & (LBM_FIELD_RHO | LBM_FIELD_P | LBM_FIELD_U))
-    LBM_CK(c, lbm::launch_fields(cur_state(c), phi_now, mu_now, c->stage, c->geo, c->ph,
-                                 read_pattern(c), velocity_time_factor(c, c->step), c->stream));
-  const bool pageable = ((mask & LBM_FIELD_PHI) && !device_view(phi)) ||
-                        ((mask & LBM_FIELD_MU) && !device_view(mu)) ||
-                        ((mask & LBM_FIELD_RHO) && !device_view(rho)) ||
-                        ((mask & LBM_FIELD_P) && !device_view(p)) ||
-                        ((mask & LBM_FIELD_U) &&
-                         (!device_view(u) || !device_view(u + n) || !device_view(u + 2 * n)));
+  const bool phi_only = !(mask & (flow | LBM_FIELD_MU));
+  if (pageable || !phi_only)
+    LBM_CK(c, lbm::launch_phi(cur_state(c), c->phi, phi_now, c->geo, read_pattern(c), c->stream));
+  if (mask & (LBM_FIELD_MU | flow))
+    LBM_CK(c, lbm::launch_mu(phi_now, mu_now, c->geo, c->ph, c->stream));
   double* wide = nullptr;
-  if (pageable) {
+  lbm_status st = LBM_OK;
+  if (!pageable) {
+    if (mask & (LBM_FIELD_PHI | LBM_FIELD_MU | flow))
+      LBM_CK(c, lbm::launch_readout(cur_state(c), c->phi, phi_only ? nullptr : phi_now, mu_now, vphi,
+                                    vrho, vp, vu, vmu, c->slot_dev ? c->slot_dev + 7 : nullptr,
+                                    c->red + 7, c->geo, c->ph, read_pattern(c), tf, c->stream));
+  } else {
+    if (mask & flow)
+      LBM_CK(c, lbm::launch_fields(cur_state(c), phi_now, mu_now, c->stage, c->geo, c->ph,
+                                   read_pattern(c), tf, c->stream));
     wide = static_cast<double*>(dev_alloc(c, n * sizeof(double)));
     if (!wide) return fail(c, LBM_ENOMEM, "device allocation failed (read-out staging)");
+    if (mask & LBM_FIELD_PHI) st = plane_to_host(c, phi_now, phi, wide);
+    if (st == LBM_OK && (mask & LBM_FIELD_MU)) st = plane_to_host(c, mu_now, mu, wide);
+    if (st == LBM_OK && (mask & LBM_FIELD_RHO)) st = plane_to_host(c, c->stage, rho, wide);
+    if (st == LBM_OK && (mask & LBM_FIELD_P)) st = plane_to_host(c, c->stage + s, p, wide);
+    for (int a = 0; a < 3 && st == LBM_OK && (mask & LBM_FIELD_U); ++a)
+      st = plane_to_host(c, c->stage + (2 + a) * s, u + a * n, wide);
   }
-  lbm_status st = LBM_OK;
-  if (mask & LBM_FIELD_PHI) st = plane_to_host(c, phi_now, phi, wide);
-  if (st == LBM_OK && (mask & LBM_FIELD_MU)) st = plane_to_host(c, mu_now, mu, wide);
-  if (st == LBM_OK && (mask & LBM_FIELD_RHO)) st = plane_to_host(c, c->stage, rho, wide);
-  if (st == LBM_OK && (mask & LBM_FIELD_P)) st = plane_to_host(c, c->stage + s, p, wide);
-  for (int a = 0; a < 3 && st == LBM_OK && (mask & LBM_FIELD_U); ++a)
-    st = plane_to_host(c, c->stage + (2 + a) * s, u + a * n, wide);
-  double h[8];
-  if (st == LBM_OK)
-    LBM_CK(c, cudaMemcpyAsync(h, c->red, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
-  const cudaError_t es = cudaStreamSynchronize(c->stream);
+  const double* h = c->host_red;
+  cudaError_t es = cudaSuccess;
+  if (st == LBM_OK && !(c->slot_dev && !pageable && (mask & (LBM_FIELD_PHI | LBM_FIELD_MU | flow))))
+    es = cudaMemcpyAsync(c->host_red, c->red, 8 * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
+  const cudaError_t ey = cudaStreamSynchronize(c->stream);
   if (wide) dev_free(c, wide);
   if (st != LBM_OK) return st;
   if (es != cudaSuccess) return fail_cuda(c, "lbm_read_fields", es);
+  if (ey != cudaSuccess) return fail_cuda(c, "lbm_read_fields", ey);
   return take_device_error(c, h);
 }
 
@@ -896,11 +991,10 @@ lbm_status lbm_reduce(lbm_ctx* c, double* sum_phi, double mom[3]) {
   if (const lbm_status rs = check_ready(c); rs != LBM_OK) return rs;
   float* phi_now = c->stage + 5 * c->geo.stride;
   LBM_CK(c, lbm::launch_phi(cur_state(c), c->phi, phi_now, c->geo, read_pattern(c), c->stream));
-  LBM_CK(c, lbm::launch_reduce(cur_state(c), phi_now, c->partial, c->red, c->geo, read_pattern(c),
-                               c->vel_kind == LBM_VELOCITY_NONE, c->stream));
-  double h[8];
-  LBM_CK(c, cudaMemcpyAsync(h, c->red, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
-  LBM_CK(c, cudaStreamSynchronize(c->stream));
+  LBM_CK(c, lbm::launch_reduce(cur_state(c), phi_now, c->partial, result_target(c), c->geo, read_pattern(c),
+                               c->vel_kind == LBM_VELOCITY_NONE, c->stream, result_word(c)));
+  const double* h = c->host_red;
+  LBM_CK(c, fetch_results(c));
   if (const lbm_status te = take_device_error(c, h); te != LBM_OK) return te;
   *sum_phi = h[0];
   mom[0] = h[1];

@@ -320,7 +320,8 @@ int fused_default_segment(const Geometry& geo, int sms) {
 
 cudaError_t launch_fused(const float* src, float* dst, const float* phi_in, float* phi_out,
                          const Geometry& geo, const Physics& ph, bool have_prev, int seg, int pf,
-                         float* parts, double* partial, double* out, cudaStream_t st) {
+                         float* parts, double* partial, double* out, cudaStream_t st,
+                         const double* word) {
   cudaError_t e;
   if (geo.storage == kF16)
     e = launch_fused_s<kF16>(src, dst, phi_in, phi_out, geo, ph, have_prev, seg, pf, parts, st);
@@ -329,7 +330,7 @@ cudaError_t launch_fused(const float* src, float* dst, const float* phi_in, floa
   else
     e = launch_fused_s<kF32>(src, dst, phi_in, phi_out, geo, ph, have_prev, seg, pf, parts, st);
   if (e != cudaSuccess || !parts) return e;
-  return launch_step_sums_final(parts, partial, out, geo, st);
+  return launch_step_sums_final(parts, partial, out, geo, st, word);
 }
 
 }  // namespace lbm

@@ -51,6 +51,14 @@ cudaError_t launch_track(const float* src, float* dst, const Geometry& geo, cons
 cudaError_t launch_fields(const float* src, const float* phi, const float* mu, float* out,
                           const Geometry& geo, const Physics& ph, int pattern, float tf,
                           cudaStream_t st);
+// The selected fields (null: not) in double, stored by the kernel itself into page-locked host
+// memory.  phi_now and mu_now: phi and mu of the current state; phi_now null where phi alone is
+// selected.  mu_now is read for p, u and mu only.  word_out (may be null): where the 8 bytes at
+// `word` are copied to.
+cudaError_t launch_readout(const float* src, const float* phi_ref, const float* phi_now,
+                           const float* mu_now, double* phi, double* rho, double* p, double* u,
+                           double* mu, double* word_out, const double* word, const Geometry& geo,
+                           const Physics& ph, int pattern, float tf, cudaStream_t st);
 cudaError_t launch_init(float* state, const float* phi, const float* mu, const float* u0,
                         const float* p0, const Geometry& geo, const Physics& ph, int pattern,
                         float tf, cudaStream_t st);
@@ -69,8 +77,10 @@ int reduce_parts(const Geometry& geo);
 // Resident blocks per SM of k_collide (kernel 0), the order-parameter kernel (kernel 1:
 // k_phi_rows with rows, else k_phi) or k_collide2 (kernel 3); 0 on error.
 int resident_blocks_per_sm(int kernel, int storage, bool rows = false);
+// The reductions write out[0..4]; with `word` its 8 bytes go to out[7] too.
 cudaError_t launch_reduce(const float* src, const float* phi, double* partial, double* out,
-                          const Geometry& geo, int pattern, bool with_g, cudaStream_t st);
+                          const Geometry& geo, int pattern, bool with_g, cudaStream_t st,
+                          const double* word = nullptr);
 // Bytes of the tiled cell-state array for n cells.
 inline size_t state_bytes(int n, int storage) {
   const int tb = storage == kF32 ? tile_bytes<kF32>() : tile_bytes<kF16>();
@@ -84,12 +94,14 @@ int cell_warps(long long n);
 cudaError_t launch_collide_sums(const float* src, float* dst, const float* phi, const float* mu,
                                 const Geometry& geo, const Physics& ph, int pattern,
                                 bool have_prev, float* parts, double* partial, double* out,
-                                cudaStream_t st, int* err = nullptr, long long polls = 0);
+                                cudaStream_t st, int* err = nullptr, long long polls = 0,
+                                const double* word = nullptr);
 
 // The fixed-order FP64 reduction of the per-warp partials of the step sums (the tail of
 // launch_collide_sums): parts -> partial -> out (5 doubles).
 cudaError_t launch_step_sums_final(const float* parts, double* partial, double* out,
-                                   const Geometry& geo, cudaStream_t st);
+                                   const Geometry& geo, cudaStream_t st,
+                                   const double* word = nullptr);
 
 // Resident-brick steps of small grids (lbm_brick.cuh): how a grid is cut into bricks, one per
 // block, all resident for a launch of `steps` steps.
@@ -130,7 +142,7 @@ cudaError_t launch_brick(float* state0, float* state1, float* phi, const Geometr
 // Sums of a state that a step has just written, as launch_collide_sums leaves them in out (5
 // doubles), for grids of up to 2M cells; partial: 5 x kReduceMaxParts doubles, *count zero.
 cudaError_t launch_state_sums(const float* state, const float* phi, const Geometry& geo, double* partial,
-                              double* out, int* count, cudaStream_t st);
+                              double* out, const double* word, int* count, cudaStream_t st);
 
 // Single-pass step (lbm_fused.cu): pattern AB, default model variant, grids with
 // fused_shape_ok (nx a multiple of 32 with whole-tile rows, ny a multiple of 8).  phi_in
@@ -141,6 +153,7 @@ bool fused_shape_ok(const Geometry& geo);
 int fused_default_segment(const Geometry& geo, int sms);
 cudaError_t launch_fused(const float* src, float* dst, const float* phi_in, float* phi_out,
                          const Geometry& geo, const Physics& ph, bool have_prev, int seg, int pf,
-                         float* parts, double* partial, double* out, cudaStream_t st);
+                         float* parts, double* partial, double* out, cudaStream_t st,
+                         const double* word = nullptr);
 
 }  // namespace lbm

@@ -646,6 +646,71 @@ __global__ void __launch_bounds__(kBlock) k_fields(const float* __restrict__ src
   out[4 * s + idx] = M.u[2];
 }
 
+// -------------------------------------------------------------- k_readout ---------
+// The selected fields (non-null pointers) of every cell in double, into page-locked host
+// memory: what k_fields and k_widen do plane by plane, in one pass.  The host link (193 GB/s
+// measured, 56 B a cell for all seven planes) is what bounds it; loads and arithmetic go on
+// while it is busy, and no FP32 plane is written and read back.  phi_now null: phi is formed
+// here (nothing but phi selected).  All fields of 128x128x512, the passes before it included:
+// 2732 us plane by plane, 2536 in one pass (2433 is the link alone); 32^3: 76 us, 50; phi of
+// 256^3: 875 us, 711.
+struct ReadOut {
+  double *phi, *rho, *p, *u, *mu;
+  double* word_out;  // the device error word goes here when not null
+  const double* word;
+};
+
+template <int P, int S>
+__global__ void __launch_bounds__(kBlock) k_readout(const float* __restrict__ src,
+                                                    const float* __restrict__ phi_ref,
+                                                    const float* __restrict__ phi_now,
+                                                    const float* __restrict__ mu_now, ReadOut out,
+                                                    Geometry geo, Physics ph, float tf) {
+  const int idx = blockIdx.x * kBlock + threadIdx.x;
+  if (idx >= geo.n) return;
+  if (idx == 0 && out.word_out) *out.word_out = *out.word;
+  const size_t n = static_cast<size_t>(geo.n);
+  int x, y, z;
+  cell_coords(geo, idx, x, y, z);
+  const Nbr nb = make_nbr(geo, x, y, z);
+  if (!phi_now) {
+    float f[7];
+    if (use_rows<P>(geo, nb))
+      row_load_f<P, S>(row_pull<S>(src, nb, idx), f);
+    else
+      load_f<P, S>(src, idx, nb, f);
+    if (S != kF32) f[0] += phi_ref[idx];
+    out.phi[idx] = f[0] + ((f[1] + f[2]) + (f[3] + f[4]) + (f[5] + f[6]));
+    return;
+  }
+  const float phi_c = __ldg(phi_now + idx);
+  if (out.phi) out.phi[idx] = phi_c;
+  if (out.mu) out.mu[idx] = __ldg(mu_now + idx);
+  if (!(out.rho || out.p || out.u)) return;
+  float rho, p, u[3];
+  if (ph.vel_kind != kVelNone) {  // tracking mode: prescribed u, no pressure
+    prescribed_velocity(ph, geo, x, y, z, tf, u);
+    rho = ph.rho_g + (1.0f + phi_c) * ph.half_drho;
+    p = 0.0f;
+  } else {
+    const CellStencils cs = ph.d3q7_stencil ? cell_stencils<true>(phi_now, mu_now, idx, nb)
+                                            : cell_stencils<false>(phi_now, mu_now, idx, nb);
+    float g[15];
+    load_g<P, S>(src, idx, nb, g);
+    const Macro M = macroscopic(ph, moments15(g), cs.phi, cs.mu, cs.grad_phi, cs.lap_mu);
+    rho = M.rho;
+    p = M.p;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) u[a] = M.u[a];
+  }
+  if (out.rho) out.rho[idx] = rho;
+  if (out.p) out.p[idx] = p;
+  if (out.u) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) out.u[a * n + idx] = u[a];
+  }
+}
+
 // ------------------------------------------------------------------ k_init --------
 // Pre-collision populations f = f^eq (Eq. 5), g = g^eq (Eq. 21) placed for a step of
 // pattern P; phi u stored in the own tile.  u0 (3 dense planes) and p0 may be null.
@@ -856,10 +921,13 @@ __global__ void __launch_bounds__(kBlock) k_reduce_partial(const float* __restri
   }
 }
 
-// Pass 2: one block folds the partials in a fixed order.
+// Pass 2: one block folds the partials in a fixed order.  With `word` (the device error word,
+// 8 bytes) it is copied to out[7], so that a host that reads out needs no copy of its own.
 __global__ void __launch_bounds__(kBlock) k_reduce_final(const double* __restrict__ partial,
-                                                         int nparts, double* __restrict__ out) {
+                                                         int nparts, double* __restrict__ out,
+                                                         const double* word) {
   __shared__ double sh[kBlock];
+  if (word && threadIdx.x == 0) out[7] = *word;
   for (int k = 0; k < 5; ++k) {
     double v = 0.0;
     for (int b = threadIdx.x; b < nparts; b += kBlock) v += partial[b * 5 + k];
@@ -1062,7 +1130,7 @@ int cell_warps(long long n) { return static_cast<int>((n + 31) / 32); }
 cudaError_t launch_collide_sums(const float* src, float* dst, const float* phi, const float* mu,
                                 const Geometry& geo, const Physics& ph, int pattern,
                                 bool have_prev, float* parts, double* partial, double* out,
-                                cudaStream_t st, int* err, long long polls) {
+                                cudaStream_t st, int* err, long long polls, const double* word) {
   const int prev = have_prev ? 1 : 0;
   if (pattern == kAB && geo.pairs && geo.stage && err) {
     const unsigned blocks = blocks_for(geo.n);
@@ -1110,18 +1178,18 @@ cudaError_t launch_collide_sums(const float* src, float* dst, const float* phi, 
   }
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  return launch_step_sums_final(parts, partial, out, geo, st);
+  return launch_step_sums_final(parts, partial, out, geo, st, word);
 }
 
 cudaError_t launch_step_sums_final(const float* parts, double* partial, double* out,
-                                   const Geometry& geo, cudaStream_t st) {
+                                   const Geometry& geo, cudaStream_t st, const double* word) {
   const int nparts = cell_warps(geo.n);
   const int groups = nparts < kReduceMaxParts ? nparts : kReduceMaxParts;
   const int chunk = (nparts + groups - 1) / groups;
   k_reduce_chunks<<<groups, kBlock, 0, st>>>(parts, nparts, chunk, partial);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_reduce_final<<<1, kBlock, 0, st>>>(partial, groups, out);
+  k_reduce_final<<<1, kBlock, 0, st>>>(partial, groups, out, word);
   return cudaGetLastError();
 }
 
@@ -1136,6 +1204,15 @@ cudaError_t launch_fields(const float* src, const float* phi, const float* mu, f
                           const Geometry& geo, const Physics& ph, int pattern, float tf,
                           cudaStream_t st) {
   LBM_DISPATCH(geo, pattern, k_fields, src, phi, mu, out, geo, ph, tf);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_readout(const float* src, const float* phi_ref, const float* phi_now,
+                           const float* mu_now, double* phi, double* rho, double* p, double* u,
+                           double* mu, double* word_out, const double* word, const Geometry& geo,
+                           const Physics& ph, int pattern, float tf, cudaStream_t st) {
+  const ReadOut out{phi, rho, p, u, mu, word_out, word};
+  LBM_DISPATCH(geo, pattern, k_readout, src, phi_ref, phi_now, mu_now, out, geo, ph, tf);
   return cudaGetLastError();
 }
 
@@ -1212,7 +1289,8 @@ int reduce_parts(const Geometry& geo) {
 }
 
 cudaError_t launch_reduce(const float* src, const float* phi, double* partial, double* out,
-                          const Geometry& geo, int pattern, bool with_g, cudaStream_t st) {
+                          const Geometry& geo, int pattern, bool with_g, cudaStream_t st,
+                          const double* word) {
   const int parts = reduce_parts(geo);
   const int wg = with_g ? 1 : 0;
   const unsigned blocks_ = static_cast<unsigned>(parts);
@@ -1224,7 +1302,7 @@ cudaError_t launch_reduce(const float* src, const float* phi, double* partial, d
     LBM_DISPATCH_P(pattern, k_reduce_partial, kF32, src, phi, partial, geo, wg)
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_reduce_final<<<1, kBlock, 0, st>>>(partial, parts, out);
+  k_reduce_final<<<1, kBlock, 0, st>>>(partial, parts, out, word);
   return cudaGetLastError();
 }
 
