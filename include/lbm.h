@@ -374,7 +374,7 @@ lbm_status lbm_destroy(lbm_ctx* ctx);
  * defaults 8 and 6 persistent blocks per SM for passes 0 and 1, one block per item for
  * pass 2.  lbm_batch_set_prefetch sets how many items ahead passes 0
  * and 2 prefetch into L2: -1 (default) one wave (the persistent grid, else SMs x
- * resident blocks), 0 off.  lbm_batch_set_split(b, cells): runs of at least `cells`
+ * resident blocks; FP32 pass 2 one item per SM), 0 off.  lbm_batch_set_split(b, cells): runs of at least `cells`
  * cells are stepped by lbm_step on their own streams instead (they fill the GPU alone,
  * and the single-run kernels take their parameters from the constant bank); the other
  * runs share the batched launches on the batch's stream, and the two overlap.  0
