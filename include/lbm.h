@@ -286,8 +286,8 @@ lbm_status lbm_write_state(lbm_ctx* ctx, const float* f, const float* g,
  * (LBM_TUNE_TMA_WAIT_POLLS, same error reporting).  lbm_get_tuning reports 1 only while
  * it applies.  Identical results.
  * LBM_TUNE_BRICKS: 1 (default) lets lbm_step and lbm_step_reduce advance small grids
- * (LBM_PATTERN_AB; up to 640,000 cells, 180,000 with 16-bit populations, 1.6 million in
- * interface-tracking mode) by one kernel per call that keeps every block on its own brick of
+ * (up to 640,000 cells, 180,000 with 16-bit populations, 1.6 million in interface-tracking
+ * mode; LBM_PATTERN_AA up to 36,000, 270,000 in interface-tracking mode) by one kernel per call that keeps every block on its own brick of
  * cells for all the steps, blocks waiting for their neighbours between steps.  The wait is
  * bounded; one that runs out is reported as LBM_ETIMEOUT like the TMA passes' waits.
  * lbm_get_tuning reports 1 only while it applies: not while profiling or with LBM_TUNE_FUSED,

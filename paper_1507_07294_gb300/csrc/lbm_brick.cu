@@ -5,13 +5,13 @@
 
 namespace lbm {
 
-const void* brick_kernel_f32(int mode, int var, bool pair);
+const void* brick_kernel_f32(int mode, int var, bool pair, bool in_place);
 cudaError_t state_sums_f32(const float* state, const float* phi, const Geometry& geo, double* partial,
                         double* out, const double* word, int* count, cudaStream_t st);
-const void* brick_kernel_f16(int mode, int var, bool pair);
+const void* brick_kernel_f16(int mode, int var, bool pair, bool in_place);
 cudaError_t state_sums_f16(const float* state, const float* phi, const Geometry& geo, double* partial,
                         double* out, const double* word, int* count, cudaStream_t st);
-const void* brick_kernel_bf16(int mode, int var, bool pair);
+const void* brick_kernel_bf16(int mode, int var, bool pair, bool in_place);
 cudaError_t state_sums_bf16(const float* state, const float* phi, const Geometry& geo, double* partial,
                         double* out, const double* word, int* count, cudaStream_t st);
 
@@ -26,13 +26,13 @@ bool brick_div_ok(int d, long long most) {
   return most * m < (1ull << 32) && most * over < (1ull << kBrickDivShift);
 }
 
-const void* kernel_of(const Geometry& geo, const Physics& ph, int mode, bool pair) {
+const void* kernel_of(const Geometry& geo, const Physics& ph, int mode, bool pair, bool in_place) {
   const int var = mode == kBrickTracking
                       ? 0
                       : (ph.srt_flow ? kVarSrtFlow : 0) | (ph.d3q7_stencil ? kVarD3Q7 : 0);
-  return geo.storage == kF16    ? brick_kernel_f16(mode, var, pair)
-         : geo.storage == kBF16 ? brick_kernel_bf16(mode, var, pair)
-                                : brick_kernel_f32(mode, var, pair);
+  return geo.storage == kF16    ? brick_kernel_f16(mode, var, pair, in_place)
+         : geo.storage == kBF16 ? brick_kernel_bf16(mode, var, pair, in_place)
+                                : brick_kernel_f32(mode, var, pair, in_place);
 }
 
 // One way to cut an axis: bricks, cells of the largest, bricks within the cells a step reads.
@@ -66,13 +66,15 @@ bool divisions_ok(const AxisCut c[3], int halo) {
 
 // The line lies where the two state arrays outgrow the L2 cache (129 MB): 640,000 cells of
 // 2 x 100 B coupled in FP32, 1.6M of 2 x 40 B in tracking mode, where f and phi u are all
-// that moves.  Measured just inside it: 96x96x64 (590k cells) 32.8 -> 28.1 us a step,
-// tracking at 116^3 (1.56M) 49.3 -> 32.9 us; beyond it (64x64x256, 1.05M cells) the bricks'
-// halos come from DRAM and the kernel takes 57-63 us where the three passes take 63.7.
-// With 16-bit populations the coupled kernel gains less (its 2-byte loads bring half as much
-// each) and the line is where it stops gaining: 56x57x55 (176k cells) 19.5 -> 13.9 us,
-// 64^3 (262k) 18.4 -> 18.5.
-long long brick_most_cells(int mode, int storage) {
+// that moves.  Measured just inside it, three passes (one in tracking mode) -> bricks:
+// 96x96x64 (590k cells) 32.6 -> 27.6 us a step, 80^3 27.7 -> 27.6, tracking at 116^3 (1.56M)
+// 41.9 -> 32.8; beyond it (64x64x256, 1.05M cells) the bricks' halos come from DRAM: 57-63 us
+// against 48.  With 16-bit populations the coupled kernel gains less (its 2-byte loads bring
+// half as much each): 56x57x55 (176k cells) 14.4 -> 13.9 us, 64^3 (262k) 18.4 -> 18.5.  In
+// place a step has two waits and the bricks pay for the smallest boxes only: 32^3 9.2 -> 8.8
+// us, 48^3 11.3 -> 11.7; tracking 64^3 19.2 -> 12.4, 80^3 20.5 -> 21.0.
+long long brick_most_cells(int mode, int storage, bool in_place) {
+  if (in_place) return mode == kBrickTracking ? 270000 : 36000;
   if (mode == kBrickTracking) return 1600000;
   return storage == kF32 ? 640000 : 180000;
 }
@@ -85,12 +87,13 @@ long long brick_most_cells(int mode, int storage) {
 // for rows that do not start on tiles; a lone block with several rounds per SM waits more.
 // Two cells per thread pay from about 1024 cells a block (64x64x128, 256 bricks of 32x8x8:
 // 24.9 us, one cell per thread 26.3); they leave room for 2 blocks an SM instead of 3.
-// Measured per step, three passes -> bricks: 16^3 12.3 -> 4.2 us, 32^3 14.3 -> 5.1,
-// 48^3 16.4 -> 7.9, 64^3 24.6 -> 13.9, 64x64x128 38.9 -> 25.1, 37x41x45 15.4 -> 8.5;
-// tracking 32^3 19.5 -> 3.8, 64^3 18.5 -> 8.0, 100^3 38.2 -> 21.3; FP16 32^3 14.4 -> 6.2.
-BrickPlan brick_plan(const Geometry& geo, const Physics& ph, int mode, int sms) {
+// Measured per step, three passes -> bricks: 16^3 9.2 -> 4.2 us, 32^3 9.2 -> 5.1, 48^3
+// 11.5 -> 7.9, 64^3 18.5 -> 13.9, 64x64x128 29.6 -> 25.1, 37x41x45 10.3 -> 8.5; tracking 48^3
+// 12.3 -> 5.6, 100^3 30.6 -> 21.3; FP16 32^3 10.2 -> 6.2.
+BrickPlan brick_plan(const Geometry& geo, const Physics& ph, int mode, bool in_place, int sms) {
   BrickPlan p{};
-  if (geo.n > brick_most_cells(mode, geo.storage) || sms < 1) return p;
+  p.in_place = in_place ? 1 : 0;
+  if (geo.n > brick_most_cells(mode, geo.storage, in_place) || sms < 1) return p;
   const int halo = mode == kBrickTracking ? 1 : 2;
   constexpr int kWant = 9;
   static const int want[2][kWant] = {{8, 12, 16, 24, 32, 48, 64, 96, 128}, {2, 3, 4, 5, 6, 8, 10, 12, 16}};
@@ -116,14 +119,14 @@ BrickPlan brick_plan(const Geometry& geo, const Physics& ph, int mode, int sms) 
           around *= std::min(a.nb, 2 * a.reach + 1);
         }
         if (mode == kBrickTracking) mu = 0;
-        const long long smem = 4 * (phi + mu + offsets);
+        const long long smem = 4 * (phi + mu + (in_place ? 0 : offsets));
         const int per = static_cast<int>((bricks + sms - 1) / sms);
         if (around > kBrickThreads || smem > kBrickSmem || per * (smem + 1024) > 226 * 1024) continue;
         for (int pair = 0; pair < 2; ++pair) {
-          if (pair && (mode == kBrickTracking || cells < 1024 || per > 2)) continue;
+          if (pair && (mode == kBrickTracking || in_place || cells < 1024 || per > 2)) continue;
           const long long round = pair ? 2 * kBrickThreads : kBrickThreads;
           const double cell = mode == kBrickTracking ? 1.2e-3 : (cells >= 1024 && !pair ? 2.9e-3 : 2.7e-3);
-          double work = 4.4e-4 * (phi + mu) + cell * ((cells + round - 1) / round * round);
+          double work = 4.4e-4 * ((in_place ? phi / 3 : phi) + mu) + cell * ((cells + round - 1) / round * round);
           work *= 1.0 + 4.0 / c[0].b;
           if (geo.row_tiles && c[0].b % 16 != 0) work *= 1.08;
           const double est = 3.65 + per * work * (per == 1 && cells > 512 ? 1.3 : 1.0);
@@ -142,7 +145,7 @@ BrickPlan brick_plan(const Geometry& geo, const Physics& ph, int mode, int sms) 
         }
       }
   if (p.nbricks == 0) return p;
-  const void* k = kernel_of(geo, ph, mode, p.pair != 0);
+  const void* k = kernel_of(geo, ph, mode, p.pair != 0, in_place);
   int per = 0;
   if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kBrickSmem) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, kBrickThreads, p.smem) != cudaSuccess ||
@@ -163,14 +166,21 @@ BrickPlan brick_plan(const Geometry& geo, const Physics& ph, int mode, int sms) 
 
 cudaError_t launch_brick(float* state0, float* state1, float* phi, const Geometry& geo,
                          const Physics& ph, const BrickPlan& plan, const BrickTimes& times, int steps,
-                         int* flags, int base, bool have_prev, int* err, long long polls,
+                         int* flags, int base, bool have_prev, bool odd, int* err, long long polls,
                          cudaStream_t st) {
   BrickPlan bp = plan;
   bp.steps = steps;
   int hp = have_prev ? 1 : 0;
+  int od = odd ? 1 : 0;
+  if (plan.in_place) {
+    void* args[] = {&state0, &phi, const_cast<Geometry*>(&geo), const_cast<Physics*>(&ph), &bp,
+                    const_cast<BrickTimes*>(&times), &flags, &base, &hp, &od, &err, &polls};
+    return cudaLaunchCooperativeKernel(kernel_of(geo, ph, plan.mode, false, true), dim3(plan.nbricks),
+                                       dim3(kBrickThreads), args, plan.smem, st);
+  }
   void* args[] = {&state0, &state1, &phi, const_cast<Geometry*>(&geo), const_cast<Physics*>(&ph), &bp,
                   const_cast<BrickTimes*>(&times), &flags, &base, &hp, &err, &polls};
-  const void* k = kernel_of(geo, ph, plan.mode, plan.pair != 0);
+  const void* k = kernel_of(geo, ph, plan.mode, plan.pair != 0, plan.in_place != 0);
   // in a single step no block waits for another, so they need not be resident together
   return steps == 1
              ? cudaLaunchKernel(k, dim3(plan.nbricks), dim3(kBrickThreads), args, plan.smem, st)

@@ -1,11 +1,11 @@
 // Many time steps of a small grid in one launch (lbm_brick_*.cu instantiate it, one storage
 // type each): the passes of lbm_kernels.cu -- order parameter (Eqs. 13, 16), chemical
 // potential (Eq. 2), stream-collide (Eqs. 14-34) -- for boxes whose two state arrays stay in
-// the L2 cache (pattern AB, n up to brick_most_cells).
+// the L2 cache (n up to brick_most_cells).
 //
 // What bounds such a box is not bandwidth but latency: three launches a step, each with a
-// ramp, a tail and one round of loads, took 13-14 us at 32^3 and 24.6 us at 64^3, of which
-// the arithmetic is 1-3 us.  Here every block keeps one brick of cells for the whole launch
+// ramp, a tail and one round of loads, take 9.2 us at 32^3 and 18.5 us at 64^3, of which the
+// arithmetic is 1-3 us.  Here every block keeps one brick of cells for the whole launch
 // (all blocks are resident: a cooperative launch) and a step costs one wait: the block
 // forms phi on its brick and two cells around it from the streamed f, mu on one cell
 // around it, both in shared memory, collides its cells and tells the blocks around it.
@@ -16,9 +16,9 @@
 // Every value is formed by the operations of the three passes in their order, so the state
 // is the same bit for bit.
 //
-// At 32^3 a step's 5.1 us (14.3 before) are the wait (0.6), the loads' issue (0.5), phi
+// At 32^3 a step's 5.1 us are the wait (0.6), the loads' issue (0.5), phi
 // (0.9), mu (0.5), the collision (1.4) and the release of the stores (0.6), as clocks read
-// in the kernel say: latency throughout.  At 64^3 (13.9 us, 24.6 before) the collision's
+// in the kernel say: latency throughout.  At 64^3 (13.9 us) the collision's
 // arithmetic is the largest part.  brick_plan has the times over the sizes.
 #pragma once
 
@@ -120,6 +120,20 @@ __device__ __forceinline__ float region_mu(const float* c, int sy, int sz, const
   return chemical_potential(ph, c1, lap);
 }
 
+// Counter of the brick that this thread waits for, of those around brick (bi, bj, bk) that lie
+// within the cells a step reads; null for the threads beyond their number.
+__device__ __forceinline__ const int* brick_neighbour(const BrickPlan& bp, const int* flags, int bi,
+                                                      int bj, int bk) {
+  const int tid = threadIdx.x;
+  if (tid >= bp.around) return nullptr;
+  const int ax = min(bp.nb[0], 2 * bp.reach[0] + 1), ay = min(bp.nb[1], 2 * bp.reach[1] + 1);
+  const int k = tid / (ax * ay), j = (tid - k * ax * ay) / ax, i = tid - (k * ay + j) * ax;
+  const int ni = wrap_near(bi - bp.reach[0] + i, bp.nb[0]);
+  const int nj = wrap_near(bj - bp.reach[1] + j, bp.nb[1]);
+  const int nk = wrap_near(bk - bp.reach[2] + k, bp.nb[2]);
+  return flags + ((nk * bp.nb[1] + nj) * bp.nb[0] + ni) * kBrickFlag;
+}
+
 // MODE: kBrickCoupled, or kBrickTracking (prescribed velocity: only f evolves, mu is needed
 // at the brick's own cells only, so the halo is one cell narrower and there is no mu region).
 // NC cells per thread at a time in the coupled collision: 1, or 2 in the lanes of paired
@@ -152,15 +166,7 @@ __global__ void __launch_bounds__(kBrickThreads, NC == 1 ? 3 : 2)
   const int dx = brick_first(bi + 1, geo.nx, bp.nb[0]) - x0,
             dy = brick_first(bj + 1, geo.ny, bp.nb[1]) - y0,
             dz = brick_first(bk + 1, geo.nz, bp.nb[2]) - z0;
-  const int* neighbour = nullptr;
-  if (tid < bp.around) {
-    const int ax = min(bp.nb[0], 2 * bp.reach[0] + 1), ay = min(bp.nb[1], 2 * bp.reach[1] + 1);
-    const int k = tid / (ax * ay), j = (tid - k * ax * ay) / ax, i = tid - (k * ay + j) * ax;
-    const int ni = wrap_near(bi - bp.reach[0] + i, bp.nb[0]);
-    const int nj = wrap_near(bj - bp.reach[1] + j, bp.nb[1]);
-    const int nk = wrap_near(bk - bp.reach[2] + k, bp.nb[2]);
-    neighbour = flags + ((nk * bp.nb[1] + nj) * bp.nb[0] + ni) * kBrickFlag;
-  }
+  const int* neighbour = brick_neighbour(bp, flags, bi, bj, bk);
 
   // byte offsets of the brick's cells and of those around it (beyond the brick's last row or
   // column, where bricks differ in size, those of the last one: never used)
@@ -395,6 +401,186 @@ __global__ void __launch_bounds__(kBrickThreads, NC == 1 ? 3 : 2)
   }
 }
 
+// The same for the in-place pattern.  A neighbour's f may already be overwritten when a halo
+// would be formed from it, so phi is passed between blocks instead of computed twice: a block
+// forms phi of its own cells, writes it and tells the blocks around it, waits for theirs, reads
+// the halo of phi, forms mu and collides -- two waits a step.  `odd`: parity of the stored
+// populations at the first step.  phi holds the order parameter of the step before (16-bit
+// storage) and of each step in turn.
+// Measured per step, three passes -> bricks: 16^3 9.2 -> 6.1 us, 32^3 9.2 -> 8.8; tracking 32^3
+// 14.4 -> 6.9, 64^3 19.2 -> 12.4.
+template <int MODE, int VAR, int S>
+__global__ void __launch_bounds__(kBrickThreads, 3)
+    k_brick_aa(float* state, float* phi, const __grid_constant__ Geometry geo,
+               const __grid_constant__ Physics ph, const __grid_constant__ BrickPlan bp,
+               const __grid_constant__ BrickTimes times, int* flags, int base, int have_prev, int odd,
+               int* err, long long polls) {
+  extern __shared__ float smem[];
+  constexpr bool TRACK = MODE == kBrickTracking;
+  constexpr bool D3Q7 = (VAR & kVarD3Q7) != 0;
+  constexpr int H = TRACK ? 1 : 2, T = kBrickThreads;
+  const int tid = threadIdx.x;
+  const int px = bp.b[0] + 2 * H, py = bp.b[1] + 2 * H;
+  const int mx = bp.b[0] + 2, my = bp.b[1] + 2;
+  float* sphi = smem;
+  float* smu = smem + px * py * (bp.b[2] + 2 * H);
+  const int br = blockIdx.x, bxy = bp.nb[0] * bp.nb[1];
+  const int bk = br / bxy, bj = (br - bk * bxy) / bp.nb[0], bi = br - bk * bxy - bj * bp.nb[0];
+  const int x0 = brick_first(bi, geo.nx, bp.nb[0]), y0 = brick_first(bj, geo.ny, bp.nb[1]),
+            z0 = brick_first(bk, geo.nz, bp.nb[2]);
+  const int dx = brick_first(bi + 1, geo.nx, bp.nb[0]) - x0,
+            dy = brick_first(bj + 1, geo.ny, bp.nb[1]) - y0,
+            dz = brick_first(bk + 1, geo.nz, bp.nb[2]) - z0;
+  const int* neighbour = brick_neighbour(bp, flags, bi, bj, bk);
+  const int nphi = px * py * (dz + 2 * H);
+  auto real_plane = [&](int l, int first) {
+    return geo.walls ? min(max(first + l, 0), geo.nz - 1) - first : l;
+  };
+  // one wait for every block around to have reached `step` (in half steps)
+  auto wait = [&](int step) {
+    bool ok = true;
+    if (neighbour) {
+      ok = false;
+      for (long long q = 0; q < polls; ++q) {
+        if (flag_load(neighbour) - base >= step) {
+          ok = true;
+          break;
+        }
+        if ((q & 63) == 63 && flag_load(err) != 0) break;
+      }
+    }
+    if (__syncthreads_and(ok)) return true;
+    if (tid == 0) atomicMax(err, 1);
+    return false;
+  };
+  const int ncell = bp.b[0] * bp.b[1] * dz;
+  struct At {
+    int idx, x, y, z, ci, cm;
+    bool in;
+  };
+  auto place = [&](int k) {
+    At a;
+    const int r = small_div(k, bp.m_bx), i = k - r * bp.b[0];
+    const int l = small_div(r, bp.m_by), j = r - l * bp.b[1];
+    a.in = k < ncell && i < dx && j < dy;
+    const int ii = min(i, dx - 1), jj = min(j, dy - 1), ll = min(l, dz - 1);
+    a.x = x0 + ii;
+    a.y = y0 + jj;
+    a.z = z0 + ll;
+    a.idx = (a.z * geo.ny + a.y) * geo.nx + a.x;
+    a.ci = ((ll + H) * py + jj + H) * px + ii + H;
+    a.cm = ((ll + 1) * my + jj + 1) * mx + ii + 1;
+    return a;
+  };
+  for (int t = 0; t < bp.steps; ++t) {
+    const bool odd_step = ((odd + t) & 1) != 0;
+    const int hp = t > 0 ? 1 : have_prev;
+    if (t > 0 && !wait(2 * t)) return;
+    // the first cells' populations are kept for their collision
+    At at = place(tid);
+    Nbr nb = make_nbr(geo, at.x, at.y, at.z);
+    float g[15], f[7], prev[3];
+    auto load = [&](const At& a, const Nbr& n) {
+      if (TRACK) {
+        odd_step ? load_f<kAAOdd, S>(state, a.idx, n, f) : load_f<kAAEven, S>(state, a.idx, n, f);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) prev[i] = state[phiu_index<S>(a.idx, i)];
+      } else if (odd_step) {
+        load_cell<kAAOdd, S, true>(state, geo, a.idx, n, g, f, prev);
+      } else {
+        load_cell<kAAEven, S, true>(state, geo, a.idx, n, g, f, prev);
+      }
+    };
+    auto own_phi = [&](const At& a, const float* v) {
+      const float f0 = S != kF32 ? v[0] + phi[a.idx] : v[0];
+      const float p = f0 + ((v[1] + v[2]) + (v[3] + v[4]) + (v[5] + v[6]));
+      if (a.in) {
+        sphi[a.ci] = p;
+        phi[a.idx] = p;
+      }
+    };
+    load(at, nb);
+    for (int k = tid + T; k - tid < ncell; k += T) {
+      const At a = place(k);
+      const Nbr n = make_nbr(geo, a.x, a.y, a.z);
+      float q[7];
+      odd_step ? load_f<kAAOdd, S>(state, a.idx, n, q) : load_f<kAAEven, S>(state, a.idx, n, q);
+      own_phi(a, q);
+    }
+    own_phi(at, f);
+    __syncthreads();
+    if (tid == 0) flag_store(flags + br * kBrickFlag, base + 2 * t + 1);
+    if (!wait(2 * t + 1)) return;
+#pragma unroll 4
+    for (int k = tid; k < nphi; k += T) {
+      const int r = small_div(k, bp.m_px), i = k - r * px;
+      const int l = small_div(r, bp.m_py), j = r - l * py;
+      if (i >= H && i < dx + H && j >= H && j < dy + H && l >= H && l < dz + H) continue;
+      const int x = wrap_near(x0 - H + min(i, dx + 2 * H - 1), geo.nx);
+      const int y = wrap_near(y0 - H + min(j, dy + 2 * H - 1), geo.ny);
+      const int z = wrap_near(z0 - H + real_plane(l, z0 - H), geo.nz);
+      sphi[k] = phi[(z * geo.ny + y) * geo.nx + x];
+    }
+    __syncthreads();
+    if (!TRACK) {
+      const int nmu = mx * my * (dz + 2);
+#pragma unroll 3
+      for (int k = tid; k < nmu; k += T) {
+        const int r = small_div(k, bp.m_mx), i = k - r * mx;
+        const int l = small_div(r, bp.m_my), j = r - l * my;
+        const float* c = sphi + ((real_plane(l, z0 - 1) + 1) * py + j + 1) * px + i + 1;
+        smu[k] = region_mu<D3Q7>(c, px, px * py, ph);
+      }
+      __syncthreads();
+    }
+    for (int k = tid; k - tid < ncell; k += T) {
+      if (k != tid) {
+        at = place(k);
+        nb = make_nbr(geo, at.x, at.y, at.z);
+        load(at, nb);
+      }
+      if (!at.in) continue;
+      if (TRACK) {
+        const float* c = sphi + at.ci;
+        const float phi_c = c[0];
+        const float mu_c = ph.d3q7_stencil ? region_mu<true>(c, px, px * py, ph)
+                                           : region_mu<false>(c, px, px * py, ph);
+        float u[3], dphiu[3];
+        prescribed_velocity(ph, geo, at.x, at.y, at.z, times.tf[t], u);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          const float cur = __fmul_rn(phi_c, u[i]);
+          dphiu[i] = hp ? __fsub_rn(cur, prev[i]) : 0.0f;
+          state[phiu_index<S>(at.idx, i)] = cur;
+        }
+        collide_d3q7<S != kF32>(ph, f, phi_c, mu_c, u, dphiu);
+        odd_step ? store_f<kAAOdd, S>(state, at.idx, nb, f) : store_f<kAAEven, S>(state, at.idx, nb, f);
+      } else {
+        auto stencils = [&] {
+          CellStencils cs;
+          Stencil st;
+          region_stencil(sphi + at.ci, px, px * py, st);
+          if (D3Q7)
+            stencil_grad7(st, cs.grad_phi);
+          else
+            stencil_grad(st, cs.grad_phi);
+          cs.phi = st.c;
+          region_stencil(smu + at.cm, mx, mx * my, st);
+          cs.lap_mu = D3Q7 ? stencil_lap7(st) : stencil_lap(st);
+          cs.mu = st.c;
+          return cs;
+        };
+        if (odd_step)
+          collide_loaded<kAAOdd, VAR, S, false>(state, geo, ph, hp, at.idx, nb, g, f, prev, stencils, nullptr);
+        else
+          collide_loaded<kAAEven, VAR, S, false>(state, geo, ph, hp, at.idx, nb, g, f, prev, stencils, nullptr);
+      }
+    }
+    __syncthreads();
+    if (tid == 0) flag_store(flags + br * kBrickFlag, base + 2 * t + 2);
+  }
+}
+
 // Sums of the state as launch_collide_sums forms them, from the post-collision values the
 // last step stored (pattern AB; with 16-bit storage phi of that step), in one launch: block b
 // sums the warps' tiles [b chunk, (b + 1) chunk) of launch_step_sums_final's first pass, the
@@ -482,9 +668,18 @@ cudaError_t state_sums(const float* state, const float* phi, const Geometry& geo
   return cudaGetLastError();
 }
 
-// The instance for (mode, variant, cells per thread) of storage S.
+// The instance for (mode, variant, cells per thread; in place) of storage S.
 template <int S>
-const void* brick_kernel(int mode, int var, bool pair) {
+const void* brick_kernel(int mode, int var, bool pair, bool in_place) {
+#define LBM_BRICK_AA(MODE, VAR) reinterpret_cast<const void*>(&k_brick_aa<MODE, VAR, S>)
+  if (in_place) {
+    if (mode == kBrickTracking) return LBM_BRICK_AA(kBrickTracking, 0);
+    return var == 0               ? LBM_BRICK_AA(kBrickCoupled, 0)
+           : var == kVarSrtFlow   ? LBM_BRICK_AA(kBrickCoupled, kVarSrtFlow)
+           : var == kVarD3Q7      ? LBM_BRICK_AA(kBrickCoupled, kVarD3Q7)
+                                  : LBM_BRICK_AA(kBrickCoupled, kVarSrtFlow | kVarD3Q7);
+  }
+#undef LBM_BRICK_AA
 #define LBM_BRICK(MODE, VAR)                                            \
   (pair ? reinterpret_cast<const void*>(&k_brick<MODE, VAR, S, 2>)      \
         : reinterpret_cast<const void*>(&k_brick<MODE, VAR, S, 1>))

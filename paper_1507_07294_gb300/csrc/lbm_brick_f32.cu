@@ -3,7 +3,9 @@
 
 namespace lbm {
 
-const void* brick_kernel_f32(int mode, int var, bool pair) { return brick_kernel<kF32>(mode, var, pair); }
+const void* brick_kernel_f32(int mode, int var, bool pair, bool in_place) {
+  return brick_kernel<kF32>(mode, var, pair, in_place);
+}
 
 cudaError_t state_sums_f32(const float* state, const float* phi, const Geometry& geo, double* partial,
                            double* out, const double* word, int* count, cudaStream_t st) {

@@ -616,7 +616,7 @@ bool brick_applies(const lbm_ctx* c, int n) {
         !fused_applies(c)))
     return false;
   // with 16-bit storage the first step reads the phi array that the last one writes
-  if (n == 1 && c->geo.storage != lbm::kF32) return false;
+  if (n == 1 && c->geo.storage != lbm::kF32 && c->params.pattern == LBM_PATTERN_AB) return false;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   return cudaStreamIsCapturing(c->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
 }
@@ -624,6 +624,7 @@ bool brick_applies(const lbm_ctx* c, int n) {
 // n steps through the resident-brick kernel; with sums_out the sums of the state after them.
 lbm_status brick_steps(lbm_ctx* c, int n, double* sums_out, const double* word = nullptr) {
   const bool tracking = c->vel_kind != LBM_VELOCITY_NONE;
+  const bool ab = c->params.pattern == LBM_PATTERN_AB;
   while (n > 0) {
     const int most = tracking ? lbm::kBrickTrackSteps : lbm::kBrickSteps;
     int k = n < most ? n : most;
@@ -638,8 +639,8 @@ lbm_status brick_steps(lbm_ctx* c, int n, double* sums_out, const double* word =
       times.tf[i] = tracking && i < k ? velocity_time_factor(c, c->step + i) : 1.0f;
     const cudaError_t e = lbm::launch_brick(
         c->pop[c->cur], c->pop[1 - c->cur], c->phi, c->geo, c->ph, c->brick, times, k,
-        c->brick_flags, c->brick_base, c->have_prev, error_word(c), lbm::mu_tma_default_polls(),
-        c->stream);
+        c->brick_flags, c->brick_base, c->have_prev, c->odd, error_word(c),
+        lbm::mu_tma_default_polls(), c->stream);
     if (e == cudaErrorCooperativeLaunchTooLarge) {
       // fewer SMs than the device has (a partition of it): the three-kernel step from here on
       cudaGetLastError();
@@ -647,8 +648,11 @@ lbm_status brick_steps(lbm_ctx* c, int n, double* sums_out, const double* word =
       return sums_out ? step_sums(c, n, sums_out, word) : lbm_step(c, n);
     }
     LBM_CK(c, e);
-    c->brick_base += k;
-    c->cur = (c->cur + k) & 1;
+    c->brick_base += ab ? k : 2 * k;
+    if (ab)
+      c->cur = (c->cur + k) & 1;
+    else
+      c->odd = c->odd != ((k & 1) != 0);
     c->have_prev = true;
     c->step += k;
     n -= k;
@@ -661,11 +665,9 @@ lbm_status brick_steps(lbm_ctx* c, int n, double* sums_out, const double* word =
 
 // The plan for the context's mode (coupled or tracking).
 void plan_bricks(lbm_ctx* c) {
-  c->brick = lbm::BrickPlan{};
-  if (c->params.pattern == LBM_PATTERN_AB)
-    c->brick = lbm::brick_plan(
-        c->geo, c->ph, c->vel_kind == LBM_VELOCITY_NONE ? lbm::kBrickCoupled : lbm::kBrickTracking,
-        c->sms);
+  c->brick = lbm::brick_plan(
+      c->geo, c->ph, c->vel_kind == LBM_VELOCITY_NONE ? lbm::kBrickCoupled : lbm::kBrickTracking,
+      c->params.pattern != LBM_PATTERN_AB, c->sms);
 }
 
 // Whether the last step of lbm_step_reduce can carry the sums (else a separate pass).
@@ -700,7 +702,7 @@ lbm_status step_sums(lbm_ctx* c, int n, double* out, const double* word) {
                                  c->vel_kind == LBM_VELOCITY_NONE, c->stream, word));
     return LBM_OK;
   }
-  if (brick_applies(c, n)) return brick_steps(c, n, out, word);
+  if (c->params.pattern == LBM_PATTERN_AB && brick_applies(c, n)) return brick_steps(c, n, out, word);
   const lbm_status st = lbm_step(c, n - 1);
   return st != LBM_OK ? st : step_once(c, out, word);
 }

@@ -116,7 +116,7 @@ enum BrickMode { kBrickCoupled = 0, kBrickTracking = 1 };
 struct BrickPlan {
   int steps;
   int nbricks;      // 0: the grid does not go through the kernel
-  int mode, pair;
+  int mode, pair, in_place;
   int nb[3], b[3];  // bricks along each axis, cells of the largest along each axis
   int reach[3];     // bricks along each axis that lie within the cells a step reads
   int around;       // bricks a block waits for
@@ -127,17 +127,18 @@ struct BrickTimes {
   float tf[kBrickTrackSteps];  // time factor of the prescribed velocity at each step of the launch
 };
 // Largest grid whose steps go through the kernel.
-long long brick_most_cells(int mode, int storage);
+long long brick_most_cells(int mode, int storage, bool in_place);
 // nbricks = 0 where the grid is too large or cannot be cut so that every block is resident.
-BrickPlan brick_plan(const Geometry& geo, const Physics& ph, int mode, int sms);
+BrickPlan brick_plan(const Geometry& geo, const Physics& ph, int mode, bool in_place, int sms);
 // flags: kBrickMax * kBrickFlag step counters, all zero before the first launch; `base` is
-// what every counter holds before this one (each launch adds its steps).  phi: order
+// what every counter holds before this one (each launch adds its steps, in place twice that).
+// In place state1 is not used and `odd` is the parity of the stored populations.  phi: order
 // parameter of the step before (16-bit storage: read, and written by the last of at least two
 // steps).  A block whose wait for its neighbours runs out after `polls` looks sets *err to 1
 // and returns, and so do the others.
 cudaError_t launch_brick(float* state0, float* state1, float* phi, const Geometry& geo,
                          const Physics& ph, const BrickPlan& plan, const BrickTimes& times, int steps,
-                         int* flags, int base, bool have_prev, int* err, long long polls,
+                         int* flags, int base, bool have_prev, bool odd, int* err, long long polls,
                          cudaStream_t st);
 // Sums of a state that a step has just written, as launch_collide_sums leaves them in out (5
 // doubles), for grids of up to 2M cells; partial: 5 x kReduceMaxParts doubles, *count zero.

@@ -26,7 +26,8 @@ def test_one_pass_equals_three(L, shape, walls, stencil, kind):
                     seed=nx + 7 * ny + nz, phi_amp=0.02)
     w.walls_z, w.stencil, w.velocity = walls, stencil, kind
     with L.Solver(w) as a, L.Solver(w, pattern="aa") as b:
-        L.lbm_set_tuning(a.ctx, L.LBM_TUNE_BRICKS, 0)
+        for s in (a, b):
+            L.lbm_set_tuning(s.ctx, L.LBM_TUNE_BRICKS, 0)
         for n in (1, 4):
             a.step(n)
             b.step(n)
