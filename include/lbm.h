@@ -291,9 +291,11 @@ lbm_status lbm_write_state(lbm_ctx* ctx, const float* f, const float* g,
  * cells for all the steps, blocks waiting for their neighbours between steps.  The wait is
  * bounded; one that runs out is reported as LBM_ETIMEOUT like the TMA passes' waits.
  * lbm_get_tuning reports 1 only while it applies: not while profiling or with LBM_TUNE_FUSED,
- * not on a stream under capture, and not after one of the parameters that choose among the
- * three-kernel step's passes (MU_TMA, GRAPHS, ROWS, CELL_PAIRS, STENCIL_STAGE,
- * TMA_WAIT_POLLS) was set, until LBM_TUNE_BRICKS is set again.  Identical results.
+ * not on a stream under capture, and not after any other parameter was set, to whatever
+ * value, until LBM_TUNE_BRICKS is set again (the others belong to the three-kernel or the
+ * single-pass step, so setting one asks for that step).  Identical results.
+ * The other parameters report what the three-kernel step (LBM_TUNE_FUSED*: the single-pass
+ * step) does on this grid; while LBM_TUNE_BRICKS reports 1, lbm_step takes neither.
  * Setting any parameter drops the captured graphs (and waits for the context's
  * stream).
  * lbm_set_tuning returns LBM_EINVAL for an unknown parameter or a value out of range. */

@@ -73,7 +73,7 @@ struct lbm_ctx {
   int brick_base = 0;
   bool brick_reset = true;
   bool use_bricks = true;
-  bool chosen_passes = false;  // the caller set a parameter of the three-kernel step since
+  bool chosen_passes = false;  // the caller set another parameter since
 
   // CUDA graphs of two consecutive steps, one per parity of the stored state (which
   // array is current, or the AA step parity, and which phi array is current), replayed
@@ -607,9 +607,9 @@ size_t brick_flag_bytes() {
   return (static_cast<size_t>(lbm::kBrickMax) * lbm::kBrickFlag + 8) * sizeof(int);
 }
 
-// Whether the next n steps go through the resident-brick kernel.  Setting a parameter that
-// chooses among the passes of the three-kernel step, or the poll budget of their copies,
-// selects that step until LBM_TUNE_BRICKS is set again.  A stream under capture takes the
+// Whether the next n steps go through the resident-brick kernel.  Every other parameter is
+// one of the three-kernel (or single-pass) step: a caller that sets one, to whatever value,
+// means that step, and gets it until LBM_TUNE_BRICKS is set again.  A stream under capture takes the
 // three-kernel step too: a replayed launch would find the step counters of its first run.
 bool brick_applies(const lbm_ctx* c, int n) {
   if (!(c->use_bricks && !c->chosen_passes && c->brick.nbricks > 0 && n > 0 && !c->profiling &&
@@ -1187,9 +1187,7 @@ lbm_status lbm_set_tuning(lbm_ctx* c, int param, int value) {
       break;
     default: return fail(c, LBM_EINVAL, "unknown tuning parameter");
   }
-  if (param == LBM_TUNE_MU_TMA || param == LBM_TUNE_GRAPHS || param == LBM_TUNE_TMA_WAIT_POLLS ||
-      param == LBM_TUNE_ROWS || param == LBM_TUNE_CELL_PAIRS || param == LBM_TUNE_STENCIL_STAGE)
-    c->chosen_passes = true;
+  if (param != LBM_TUNE_BRICKS) c->chosen_passes = true;
   cudaStreamSynchronize(c->stream);  // a replay may still be running
   drop_graphs(c);                    // their kernel arguments may have changed
   return LBM_OK;

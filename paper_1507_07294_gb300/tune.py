@@ -55,6 +55,7 @@ def autotune(ctx, steps: int = 16, warm: int = 2,
     steps) and k_phi; returns, per parameter, the chosen value and the mean kernel time
     of every candidate (ms)."""
     out = {}
+    bricks = L.lbm_get_tuning(ctx, L.LBM_TUNE_BRICKS)
     for name, param, kernel, sums in TUNED:
         base = L.lbm_get_tuning(ctx, param)
         cands = sorted({int(round(f * base)) for f in fractions})
@@ -65,6 +66,8 @@ def autotune(ctx, steps: int = 16, warm: int = 2,
         best = min(times, key=times.get)
         L.lbm_set_tuning(ctx, param, best)
         out[name] = {"value": best, "default": base, "ms": {str(k): round(t, 5) for k, t in times.items()}}
+    if bricks:  # setting a distance has put them off
+        L.lbm_set_tuning(ctx, L.LBM_TUNE_BRICKS, 1)
     return out
 
 
