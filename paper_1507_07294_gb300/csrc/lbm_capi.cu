@@ -640,7 +640,7 @@ lbm_status brick_steps(lbm_ctx* c, int n, double* sums_out, const double* word =
     const cudaError_t e = lbm::launch_brick(
         c->pop[c->cur], c->pop[1 - c->cur], c->phi, c->geo, c->ph, c->brick, times, k,
         c->brick_flags, c->brick_base, c->have_prev, c->odd, error_word(c),
-        lbm::mu_tma_default_polls(), c->stream);
+        c->tma_polls < 0 ? lbm::mu_tma_default_polls() : c->tma_polls, c->stream);
     if (e == cudaErrorCooperativeLaunchTooLarge) {
       // fewer SMs than the device has (a partition of it): the three-kernel step from here on
       cudaGetLastError();
