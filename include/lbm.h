@@ -237,12 +237,14 @@ lbm_status lbm_write_state(lbm_ctx* ctx, const float* f, const float* g,
 /* Tuning parameters (no effect on results, only on speed).
  * LBM_TUNE_PREFETCH_COLLIDE / LBM_TUNE_PREFETCH_PHI: how many thread blocks ahead the
  * fused stream-collide kernel / the order-parameter kernel prefetch cell data into L2
- * (0 disables).  Default, set by lbm_create: one wave, the number of SMs times the
- * kernel's resident blocks per SM; for the FP32 stream-collide kernel a quarter of that
- * with staged stencils, half without.  LBM_TUNE_PREFETCH_COLLIDE_SUMS: the same distance
+ * (0 disables).  Default: one wave, the number of SMs times the kernel's resident blocks
+ * per SM; for the FP32 stream-collide kernel a quarter of that (LBM_PATTERN_AA: half) with
+ * staged stencils, half (two thirds) with two cells per thread, three quarters (one wave)
+ * with one.  LBM_TUNE_CELL_PAIRS and LBM_TUNE_STENCIL_STAGE, which choose among these, set
+ * it anew unless the caller has set it.  LBM_TUNE_PREFETCH_COLLIDE_SUMS: the same distance
  * for the stream-collide kernel of the last step of lbm_step_reduce and
  * lbm_step_reduce_async, which also sums the state it writes and has its own best
- * distance (default: that of LBM_TUNE_PREFETCH_COLLIDE at creation).
+ * distance (default: that of LBM_TUNE_PREFETCH_COLLIDE).
  * LBM_TUNE_MU_TMA: 1 (default) lets the chemical-potential pass fetch its halo bricks
  * with TMA tensor copies, 0 uses plain loads; the TMA path exists when nx is a multiple
  * of 32 (and >= 40), ny a multiple of 8 (10 to 524280) and nz is 18 to 1048560, and

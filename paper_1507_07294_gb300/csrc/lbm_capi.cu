@@ -58,6 +58,7 @@ struct lbm_ctx {
   int pairs = 0;             // Geometry::pairs when LBM_TUNE_CELL_PAIRS is on
   int stage_rows = 0;        // Geometry::stage when LBM_TUNE_STENCIL_STAGE is on
   int prefetch_sums = 0;     // Geometry::prefetch_collide of the steps that sum their result
+  bool own_prefetch = false, own_prefetch_sums = false;  // the caller has set that distance
 
   // single-pass step (lbm_fused.cu): enabled, planes per segment (0: by grid size), L2
   // prefetch distance in planes
@@ -663,6 +664,28 @@ lbm_status brick_steps(lbm_ctx* c, int n, double* sums_out, const double* word =
   return LBM_OK;
 }
 
+// Default L2 prefetch distance of the stream-collide pass as it is set now, in blocks: parts of
+// a wave of resident blocks.  The 16-bit pass, which waits on latency more than on bandwidth,
+// prefetches a whole wave ahead.  The FP32 pass moves 50 KB a block, and what it prefetches a
+// wave ahead is partly gone again when it is read, the sooner the better its loads are covered
+// otherwise.  Measured, us a step at the part taken (at a whole wave):
+//   two arrays, staged stencils  1/4  256x256x1024 2331 (2579), 128x128x512 313 (335)
+//   in place, staged             1/2  256x256x1024 2354 (2405), 256^3 609 (623); 1/4 2382, 617
+//   two arrays, two cells        1/2  192x256x1024 1776 (1875), 320x256x256 767 (783)
+//   in place, two cells          2/3  320x256x256 783 (795), 256x256x1024 2402 (2438); 1/2 862, 2440
+//   two arrays, one cell         3/4  250x260x1000 2345 (2366), 300^3 1023 (1022), 150x141x601 469 (474);
+//                                     1/2 2447, 1088, 468
+//   in place, one cell           1    300^3 1058; 3/4 1112
+int collide_distance(const lbm_ctx* c) {
+  const bool f32 = c->geo.storage == lbm::kF32;
+  const bool pairs = (f32 ? c->geo.pairs : c->pairs) != 0, ab = c->params.pattern == LBM_PATTERN_AB;
+  const int wave = c->sms * lbm::resident_blocks_per_sm(pairs ? 3 : 0, c->geo.storage);
+  if (!f32) return wave;
+  if (!pairs) return ab ? wave * 3 / 4 : wave;
+  if (c->geo.stage) return ab ? wave / 4 : wave / 2;
+  return ab ? wave / 2 : wave * 2 / 3;
+}
+
 // The plan for the context's mode (coupled or tracking).
 void plan_bricks(lbm_ctx* c) {
   c->brick = lbm::brick_plan(
@@ -752,32 +775,16 @@ lbm_status lbm_create(const lbm_grid* grid, const lbm_params* params, const lbm_
   // on by default with FP32 populations only: with 16-bit ones the pass is faster
   // loading its stencils per cell (the block waits for all its rows before computing)
   c->geo.stage = params->storage == LBM_STORAGE_FP32 ? c->stage_rows : 0;
-  // L2 prefetch distances, in parts of a wave of resident blocks.  The order-parameter pass
-  // and the 16-bit stream-collide, which waits on latency more than on bandwidth, prefetch a
-  // whole wave ahead.  The FP32 stream-collide moves 50 KB a block, and what it prefetches a
-  // wave ahead is partly gone again when it is read: one block per SM ahead is best with
-  // staged stencils (256x256x1024: 1935 us, a wave 2177; 128x128x512: 250, 271), half a wave
-  // without (256x256x256: 493, a wave 509, a quarter 533; 150x141x601: 371, 376, 376).
-  {
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess) {
-      const int wave = sms * lbm::resident_blocks_per_sm(c->geo.pairs ? 3 : 0, c->geo.storage);
-      c->geo.prefetch_collide = c->geo.storage != lbm::kF32 ? wave
-                                : c->geo.stage              ? wave / 4
-                                                            : wave / 2;
-      c->prefetch_sums = c->geo.prefetch_collide;
-      c->geo.prefetch_phi =
-          sms * lbm::resident_blocks_per_sm(1, c->geo.storage, c->geo.row_tiles > 0);
-    }
-  }
-  c->ph = make_physics(*params);
   {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
       c->sms = 0;
   }
+  c->geo.prefetch_collide = c->prefetch_sums = collide_distance(c);
+  c->geo.prefetch_phi =
+      c->sms * lbm::resident_blocks_per_sm(1, c->geo.storage, c->geo.row_tiles > 0);
+  c->ph = make_physics(*params);
 
   const size_t plane = c->geo.stride * sizeof(float);
   const size_t state_bytes = lbm::state_bytes(c->geo.n, c->geo.storage);
@@ -1144,9 +1151,15 @@ lbm_status lbm_set_tuning(lbm_ctx* c, int param, int value) {
   if (!c) return LBM_EINVAL;
   if (value < 0) return fail(c, LBM_EINVAL, "tuning values must be >= 0");
   switch (param) {
-    case LBM_TUNE_PREFETCH_COLLIDE: c->geo.prefetch_collide = value; break;
+    case LBM_TUNE_PREFETCH_COLLIDE:
+      c->geo.prefetch_collide = value;
+      c->own_prefetch = true;
+      break;
     case LBM_TUNE_PREFETCH_PHI: c->geo.prefetch_phi = value; break;
-    case LBM_TUNE_PREFETCH_COLLIDE_SUMS: c->prefetch_sums = value; break;
+    case LBM_TUNE_PREFETCH_COLLIDE_SUMS:
+      c->prefetch_sums = value;
+      c->own_prefetch_sums = true;
+      break;
     case LBM_TUNE_MU_TMA:
       if (value > 1) return fail(c, LBM_EINVAL, "LBM_TUNE_MU_TMA takes 0 or 1");
       c->use_phi_map = value == 1;
@@ -1188,6 +1201,10 @@ lbm_status lbm_set_tuning(lbm_ctx* c, int param, int value) {
     default: return fail(c, LBM_EINVAL, "unknown tuning parameter");
   }
   if (param != LBM_TUNE_BRICKS) c->chosen_passes = true;
+  if (param == LBM_TUNE_CELL_PAIRS || param == LBM_TUNE_STENCIL_STAGE) {  // another kernel
+    if (!c->own_prefetch) c->geo.prefetch_collide = collide_distance(c);
+    if (!c->own_prefetch_sums) c->prefetch_sums = collide_distance(c);
+  }
   cudaStreamSynchronize(c->stream);  // a replay may still be running
   drop_graphs(c);                    // their kernel arguments may have changed
   return LBM_OK;
