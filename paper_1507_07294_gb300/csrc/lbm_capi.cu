@@ -500,10 +500,10 @@ lbm_status step_once(lbm_ctx* c, double* sums_out, const double* word = nullptr)
     return LBM_OK;
   }
   if (c->vel_kind != LBM_VELOCITY_NONE && c->params.pattern == LBM_PATTERN_AB &&
-      lbm::track_shape_ok(c->geo)) {
+      lbm::track_shape_ok(c->geo, c->sms)) {
     const float tf = velocity_time_factor(c, c->step);
     LBM_CK(c, timed(c, 2, [&] {
-             return lbm::launch_track(src, dst, c->geo, c->ph, c->have_prev, tf, c->stream);
+             return lbm::launch_track(src, dst, c->geo, c->ph, c->have_prev, tf, c->sms, c->stream);
            }));
     c->cur = 1 - c->cur;
     c->have_prev = true;

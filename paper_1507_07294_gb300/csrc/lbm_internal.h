@@ -44,10 +44,10 @@ cudaError_t launch_che(const float* src, float* dst, const float* phi, const flo
                        const Geometry& geo, const Physics& ph, int pattern, bool have_prev,
                        float tf, cudaStream_t st);
 // One-pass tracking step (lbm_track.cu): phi, mu and launch_che's collision in one kernel,
-// pattern AB, for grids with track_shape_ok.
-bool track_shape_ok(const Geometry& geo);
+// pattern AB, for grids with track_shape_ok; sms: SMs of the device.
+bool track_shape_ok(const Geometry& geo, int sms);
 cudaError_t launch_track(const float* src, float* dst, const Geometry& geo, const Physics& ph,
-                         bool have_prev, float tf, cudaStream_t st);
+                         bool have_prev, float tf, int sms, cudaStream_t st);
 cudaError_t launch_fields(const float* src, const float* phi, const float* mu, float* out,
                           const Geometry& geo, const Physics& ph, int pattern, float tf,
                           cudaStream_t st);

@@ -23,7 +23,7 @@ struct TrackPlan {
   unsigned m_px, m_py, m_bx, m_by;
 };
 
-// Grids of any shape: a block takes a brick of at most 32 x 8 x 8 cells, phi on it and one cell
+// Grids of other shapes (columns_suit): a block takes a brick of at most 32 x 8 x 8 cells, phi on it and one cell
 // around it from the pulled f, then mu and the collision of its cells, whose f it pulls again
 // (from L1 and L2).
 __global__ void __launch_bounds__(kTrackThreads, 4)
@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(kTrackThreads, 4)
   }
 }
 
-// The same step for grids whose rows are whole tiles: a block marches up z through a column of
+// The same step for grids whose rows are whole tiles, where columns_suit: a block marches up z through a column of
 // 32 x 8 cells, one warp per row, two more for the rows beside the column and one for the
 // cells beside each row.  In iteration z the
 // loads of plane z + 2 are issued, phi of plane z + 1 goes to a ring in shared memory and plane
@@ -300,10 +300,50 @@ __global__ void __launch_bounds__(kColThreads, 2)
   }
 }
 
+// How k_track cuts an axis of n cells into bricks of at most `want`.
+void cut(int n, int want, int& nb, int& b) {
+  nb = (n + want - 1) / want;
+  b = (n + nb - 1) / nb;
+}
+
+// Whether the columns of k_track_rows suit the grid.  A block marches through its 32 planes one
+// after the other, so there have to be as many blocks as SMs, or few planes; columns that hang
+// over the grid's last row waste their warps.  Measured, us a step, columns (bricks): 32^3 24.6
+// (8.3), 64x33x64 26.8 (14.4), 64x64x400 62 (68); with 5 of 8 rows used 96x5x3541, 333 blocks,
+// 56 (45), 96x5x8333 94 (92), 96x5x25000 241 (258); 4 of 8 92.4 (98.3) at 32x4x31250.
+bool columns_suit(const Geometry& geo, int sms) {
+  const long long segments = (geo.nz + kColSeg - 1) / kColSeg;
+  if (geo.row_tiles == 0 || segments > 65535) return false;
+  if (geo.nz <= 8) return true;
+  const int across = (geo.ny + kColY - 1) / kColY;
+  const long long blocks = segments * across * geo.row_tiles;
+  if (geo.ny <= kColY / 2 || blocks < sms) return false;
+  // two blocks an SM: between one wave and 1.4 a mostly empty second one is worth it only for
+  // columns that are nearly full
+  return 4 * geo.ny >= 3 * kColY * across || blocks <= 2 * sms || 5 * blocks >= 14 * sms;
+}
+
 }  // namespace
 
-bool track_shape_ok(const Geometry& geo) {
-  return geo.storage == kF32 && (geo.nz + kColSeg - 1) / kColSeg <= 65535;
+// Bricks of few cells (grids thin in two directions) cost more than three passes, whose
+// order-parameter and collision passes do not care about the shape, unless the grid fills less
+// than half a dozen blocks an SM.  The line is the crossing of two fitted costs in ns a cell:
+// bricks 6.5 / (cells of a brick) + 0.019, three passes 8.5 / (cells of a chemical-potential
+// block) + 0.0225.  Measured, us a step, three passes (bricks): 8x1x750000 500 (923), 5x2x170000
+// 134 (193), 500x2x6000 170 (200), 256x1x15625 146 (164), 8x1x12500 21 (18), 8x53125x4 120 (72),
+// 100x4x15000 156 (160), 500x4x3000 148 (138).
+bool track_shape_ok(const Geometry& geo, int sms) {
+  if (geo.storage != kF32) return false;
+  if (columns_suit(geo, sms)) return true;
+  const int n[3] = {geo.nx, geo.ny, geo.nz}, want[3] = {32, 8, 8}, mu[3] = {32, 8, 16};
+  double brick = 1.0, block = geo.n;
+  for (int a = 0; a < 3; ++a) {
+    int nb, b;
+    cut(n[a], want[a], nb, b);
+    brick *= b;
+    block /= (n[a] + mu[a] - 1) / mu[a];
+  }
+  return geo.n <= 21.0 * sms * brick || 6.5 / brick < 8.5 / block + 0.0035;
 }
 
 // Rows of whole tiles march up columns in segments of 32 planes (a segment forms phi on one
@@ -311,9 +351,9 @@ bool track_shape_ok(const Geometry& geo) {
 // (0: 322, 3: 291, 8: 293); other grids take bricks (150^3: 32x8x8 75.9 us, 64x8x4 78.5,
 // 32x16x8 81.4).
 cudaError_t launch_track(const float* src, float* dst, const Geometry& geo, const Physics& ph,
-                         bool have_prev, float tf, cudaStream_t st) {
+                         bool have_prev, float tf, int sms, cudaStream_t st) {
   const int prev = have_prev ? 1 : 0;
-  if (geo.row_tiles > 0) {
+  if (columns_suit(geo, sms)) {
     const dim3 grid(geo.row_tiles * ((geo.ny + kColY - 1) / kColY), (geo.nz + kColSeg - 1) / kColSeg);
     k_track_rows<<<grid, kColThreads, 0, st>>>(src, dst, geo, ph, geo.row_tiles, prev, tf);
     return cudaGetLastError();
@@ -322,8 +362,7 @@ cudaError_t launch_track(const float* src, float* dst, const Geometry& geo, cons
   const int n[3] = {geo.nx, geo.ny, geo.nz}, want[3] = {32, 8, 8};
   long long bricks = 1;
   for (int a = 0; a < 3; ++a) {
-    p.nb[a] = (n[a] + want[a] - 1) / want[a];
-    p.b[a] = (n[a] + p.nb[a] - 1) / p.nb[a];
+    cut(n[a], want[a], p.nb[a], p.b[a]);
     bricks *= p.nb[a];
   }
   // exact for the numbers of a brick: k (m d - 2^kBrickDivShift) < 3400 * 34 < 2^kBrickDivShift
