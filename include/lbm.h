@@ -298,6 +298,12 @@ lbm_status lbm_write_state(lbm_ctx* ctx, const float* f, const float* g,
  * not on a stream under capture, and not after any other parameter was set, to whatever
  * value, until LBM_TUNE_BRICKS is set again (the others belong to the three-kernel or the
  * single-pass step, so setting one asks for that step).  Identical results.
+ * A launch of bricks starts when all its blocks fit on the device at once.  So contexts alive
+ * on several streams of a device, which may step at the same time, take the three-kernel step
+ * instead (and LBM_TUNE_BRICKS reports 0) while the fullest launch of each stream together
+ * need more room than there is, but for boxes so small that four launches fit (some 16^3;
+ * tracking: three); lbm_batch steps many runs together.  Behind other kernels that hold SMs
+ * the launch waits: set LBM_TUNE_BRICKS to 0 where such a kernel itself waits for these steps.
  * The other parameters report what the three-kernel step (LBM_TUNE_FUSED*: the single-pass
  * step) does on this grid; while LBM_TUNE_BRICKS reports 1, lbm_step takes neither.
  * Setting any parameter drops the captured graphs (and waits for the context's

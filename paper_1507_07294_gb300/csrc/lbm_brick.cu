@@ -162,6 +162,7 @@ BrickPlan brick_plan(const Geometry& geo, const Physics& ph, int mode, bool in_p
     cudaGetLastError();
     return BrickPlan{};
   }
+  p.slots = per * sms;
   p.m_qx = brick_div(p.b[0] + 2 * halo + 2);
   p.m_qy = brick_div(p.b[1] + 2 * halo + 2);
   p.m_px = brick_div(p.b[0] + 2 * halo);

@@ -7,9 +7,12 @@
 
 #include <cstdint>
 
+#include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <map>
 #include <mutex>
 #include <string>
 #include <utility>
@@ -27,6 +30,7 @@ struct lbm_ctx {
   lbm_allocator alloc{};
   bool have_alloc = false;
   cudaStream_t stream = nullptr;
+  int device = 0;
 
   // device memory
   float* pop[2] = {nullptr, nullptr};  // tiled cell state(s): 22 populations + phi u
@@ -75,6 +79,9 @@ struct lbm_ctx {
   bool brick_reset = true;
   bool use_bricks = true;
   bool chosen_passes = false;  // the caller set another parameter since
+  double part = 0.0;           // of the device that a launch takes (Sharers)
+  mutable bool room = true;    // whether that goes with the other streams' launches, as of
+  mutable unsigned room_version = 0;
 
   // CUDA graphs of two consecutive steps, one per parity of the stored state (which
   // array is current, or the AA step parity, and which phi array is current), replayed
@@ -173,6 +180,37 @@ void give_red_slot(double* slot) {
   g_red_slots.used &= ~(1ull << ((slot - g_red_slots.page) / 8));
 }
 
+// Who shares the device.  A launch of resident bricks starts when all its blocks fit at once, so
+// two of them on two streams that do not fit together take turns, where the short launches of
+// the three-kernel step overlap.  Contexts on distinct streams are taken to step at the same
+// time, those of one stream in turn: bricks_have_room where the fullest launches of all streams
+// fit the device together, or this context's is so small that four (tracking, and single
+// steps, whose blocks do not wait for one another: three) do.
+// Measured, us a step and context with K contexts on K streams, bricks (three kernels): 32^3,
+// 128 of 456 blocks: K = 2 3.3 (5.3), 4 2.8 (3.2), 8 2.8 (2.0); 48^3, 432 blocks: 2 8.1 (8.0), 8
+// 8.1 (5.3); 64^3: 2 17.3 (14.0), 8 18.4 (10.6); 16^3, 64 blocks: 8 0.9 (1.9).
+struct Sharers {
+  struct Entry {
+    int device;
+    cudaStream_t stream;
+    double part;  // of the device's slots that the context's launch takes
+  };
+  std::mutex lock;
+  std::map<const lbm_ctx*, Entry> live;
+  std::atomic<unsigned> version{1};  // counts changes of `live`
+};
+Sharers g_sharers;
+
+// Sets or (part 0) takes back the part of the device that the context's bricks take.
+void share(lbm_ctx* c, double part) {
+  std::lock_guard<std::mutex> hold(g_sharers.lock);
+  if (part > 0.0)
+    g_sharers.live[c] = {c->device, c->stream, part};
+  else if (!g_sharers.live.erase(c))
+    return;
+  g_sharers.version.fetch_add(1);
+}
+
 bool rate_ok(double s) { return s > 0.0 && s < 2.0 && std::isfinite(s); }
 
 // Multiplier and shift of the multiply-shift division by d (see lbm::FastDiv).
@@ -251,6 +289,7 @@ void drop_graphs(lbm_ctx* c) {
 }
 
 void release(lbm_ctx* c) {
+  share(c, 0.0);
   drop_graphs(c);
   if (c->capture_stream) cudaStreamDestroy(c->capture_stream);
   c->capture_stream = nullptr;
@@ -608,6 +647,31 @@ size_t brick_flag_bytes() {
   return (static_cast<size_t>(lbm::kBrickMax) * lbm::kBrickFlag + 8) * sizeof(int);
 }
 
+// What the context's bricks take of the device, as its settings are now.
+void publish_part(lbm_ctx* c) {
+  const bool on = c->use_bricks && !c->chosen_passes && c->brick.nbricks > 0;
+  c->part = on ? static_cast<double>(c->brick.nbricks) / c->brick.slots : 0.0;
+  share(c, c->part);
+}
+
+bool bricks_have_room(const lbm_ctx* c, int n) {
+  if (c->part <= (n > 1 && c->vel_kind == LBM_VELOCITY_NONE ? 1.0 / 4 : 1.0 / 3)) return true;
+  if (c->room_version != g_sharers.version.load()) {
+    std::lock_guard<std::mutex> hold(g_sharers.lock);
+    std::map<cudaStream_t, double> fullest;
+    for (const auto& e : g_sharers.live)
+      if (e.second.device == c->device) {
+        double& part = fullest[e.second.stream];
+        part = std::max(part, e.second.part);
+      }
+    double sum = 0.0;
+    for (const auto& e : fullest) sum += e.second;
+    c->room = sum <= 1.0;
+    c->room_version = g_sharers.version.load();
+  }
+  return c->room;
+}
+
 // Whether the next n steps go through the resident-brick kernel.  Every other parameter is
 // one of the three-kernel (or single-pass) step: a caller that sets one, to whatever value,
 // means that step, and gets it until LBM_TUNE_BRICKS is set again.  A stream under capture takes the
@@ -618,6 +682,7 @@ bool brick_applies(const lbm_ctx* c, int n) {
     return false;
   // with 16-bit storage the first step reads the phi array that the last one writes
   if (n == 1 && c->geo.storage != lbm::kF32 && c->params.pattern == LBM_PATTERN_AB) return false;
+  if (!bricks_have_room(c, n)) return false;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   return cudaStreamIsCapturing(c->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
 }
@@ -646,6 +711,7 @@ lbm_status brick_steps(lbm_ctx* c, int n, double* sums_out, const double* word =
       // fewer SMs than the device has (a partition of it): the three-kernel step from here on
       cudaGetLastError();
       c->brick = lbm::BrickPlan{};
+      publish_part(c);
       return sums_out ? step_sums(c, n, sums_out, word) : lbm_step(c, n);
     }
     LBM_CK(c, e);
@@ -775,12 +841,9 @@ lbm_status lbm_create(const lbm_grid* grid, const lbm_params* params, const lbm_
   // on by default with FP32 populations only: with 16-bit ones the pass is faster
   // loading its stencils per cell (the block waits for all its rows before computing)
   c->geo.stage = params->storage == LBM_STORAGE_FP32 ? c->stage_rows : 0;
-  {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      c->sms = 0;
-  }
+  if (cudaGetDevice(&c->device) != cudaSuccess ||
+      cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess)
+    c->sms = 0;
   c->geo.prefetch_collide = c->prefetch_sums = collide_distance(c);
   c->geo.prefetch_phi =
       c->sms * lbm::resident_blocks_per_sm(1, c->geo.storage, c->geo.row_tiles > 0);
@@ -825,6 +888,7 @@ lbm_status lbm_create(const lbm_grid* grid, const lbm_params* params, const lbm_
     else
       give_red_slot(slot);
   }
+  publish_part(c);
   *out = c;
   return LBM_OK;
 }
@@ -1144,6 +1208,7 @@ lbm_status lbm_set_velocity(lbm_ctx* c, int kind, double U, double period) {
   c->ph.vel_kind = kind;
   c->ph.vel_U = static_cast<float>(U);
   plan_bricks(c);
+  publish_part(c);
   return LBM_OK;
 }
 
@@ -1201,6 +1266,7 @@ lbm_status lbm_set_tuning(lbm_ctx* c, int param, int value) {
     default: return fail(c, LBM_EINVAL, "unknown tuning parameter");
   }
   if (param != LBM_TUNE_BRICKS) c->chosen_passes = true;
+  publish_part(c);
   if (param == LBM_TUNE_CELL_PAIRS || param == LBM_TUNE_STENCIL_STAGE) {  // another kernel
     if (!c->own_prefetch) c->geo.prefetch_collide = collide_distance(c);
     if (!c->own_prefetch_sums) c->prefetch_sums = collide_distance(c);

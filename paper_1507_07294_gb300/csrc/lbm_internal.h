@@ -116,6 +116,7 @@ enum BrickMode { kBrickCoupled = 0, kBrickTracking = 1 };
 struct BrickPlan {
   int steps;
   int nbricks;      // 0: the grid does not go through the kernel
+  int slots;        // blocks that the device holds at once
   int mode, pair, in_place;
   int nb[3], b[3];  // bricks along each axis, cells of the largest along each axis
   int reach[3];     // bricks along each axis that lie within the cells a step reads
