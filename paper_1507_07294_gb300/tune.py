@@ -13,12 +13,14 @@ from typing import Dict, Iterable, Optional
 
 from . import lbm as L
 
-# candidate distances as fractions of the default (one wave of resident blocks)
-DEFAULT_FRACTIONS = (0.0, 0.33, 0.5, 0.67, 0.83, 1.0, 1.17)
+# candidate distances as fractions of the default, which is a wave of resident blocks, or as
+# little as a quarter of one: up to a wave in either case
+DEFAULT_FRACTIONS = (0.0, 0.33, 0.5, 0.67, 0.83, 1.0, 1.17, 1.33, 2.0, 2.67, 3.33, 4.0)
 
 
-def _time_kernel(ctx, kernel: int, steps: int, warm: int, sums: bool = False) -> float:
-    """Mean duration (ms) of `kernel` over `steps` steps after `warm` untimed ones; with
+def _time_kernel(ctx, kernel: int, steps: int, warm: int, sums: bool = False) -> Optional[float]:
+    """Mean duration (ms) of `kernel` over `steps` steps after `warm` untimed ones, None where
+    the steps do not launch it (interface tracking in one pass, the single-pass step); with
     sums, steps that also sum their result (lbm_step_reduce_async, one step per call,
     back to back as a run that checks every step enqueues them)."""
     L.lbm_step(ctx, warm)
@@ -41,7 +43,7 @@ def _time_kernel(ctx, kernel: int, steps: int, warm: int, sums: bool = False) ->
     L.lbm_step(ctx, steps)
     ms, n = L.lbm_profile_read(ctx, kernel)
     L.lbm_profile(ctx, False)
-    return ms / max(n, 1)
+    return ms / n if n else None
 
 
 TUNED = (("prefetch_collide", L.LBM_TUNE_PREFETCH_COLLIDE, L.KERNEL_COLLIDE, False),
@@ -53,7 +55,8 @@ def autotune(ctx, steps: int = 16, warm: int = 2,
              fractions: Iterable[float] = DEFAULT_FRACTIONS) -> Dict[str, dict]:
     """Pick the fastest prefetch distance for k_collide (of plain steps and of summing
     steps) and k_phi; returns, per parameter, the chosen value and the mean kernel time
-    of every candidate (ms)."""
+    of every candidate (ms).  A parameter whose kernel the steps do not launch keeps its value
+    (and has no times)."""
     out = {}
     bricks = L.lbm_get_tuning(ctx, L.LBM_TUNE_BRICKS)
     for name, param, kernel, sums in TUNED:
@@ -62,8 +65,10 @@ def autotune(ctx, steps: int = 16, warm: int = 2,
         times = {}
         for v in cands:
             L.lbm_set_tuning(ctx, param, v)
-            times[v] = _time_kernel(ctx, kernel, steps, warm, sums)
-        best = min(times, key=times.get)
+            t = _time_kernel(ctx, kernel, steps, warm, sums)
+            if t is not None:
+                times[v] = t
+        best = min(times, key=times.get) if times else base
         L.lbm_set_tuning(ctx, param, best)
         out[name] = {"value": best, "default": base, "ms": {str(k): round(t, 5) for k, t in times.items()}}
     if bricks:  # setting a distance has put them off
