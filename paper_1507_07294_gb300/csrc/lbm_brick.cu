@@ -89,7 +89,8 @@ long long brick_most_cells(int mode, int storage, bool in_place) {
 // of threads, more for short rows (a region row of 20 touches as many lines as one of 36) and
 // for rows that do not start on tiles; a lone block with several rounds per SM waits more.
 // Two cells per thread pay from about 1024 cells a block (64x64x128, 256 bricks of 32x8x8:
-// 24.9 us, one cell per thread 26.3); they leave room for 2 blocks an SM instead of 3.
+// 24.9 us, one cell per thread 26.3); they leave room for 2 blocks an SM instead of 3.  Boxes
+// with 16-bit populations are too small for that: none of 19,671 sampled ones took it.
 // Measured per step, three passes -> bricks: 16^3 9.2 -> 4.2 us, 32^3 9.2 -> 5.1, 48^3
 // 11.5 -> 7.9, 64^3 18.5 -> 13.9, 64x64x128 29.6 -> 25.1, 37x41x45 10.3 -> 8.5; tracking 48^3
 // 12.3 -> 5.6, 100^3 30.6 -> 21.3; FP16 32^3 10.2 -> 6.2.
@@ -126,7 +127,8 @@ BrickPlan brick_plan(const Geometry& geo, const Physics& ph, int mode, bool in_p
         const int per = static_cast<int>((bricks + sms - 1) / sms);
         if (around > kBrickThreads || smem > kBrickSmem || per * (smem + 1024) > 226 * 1024) continue;
         for (int pair = 0; pair < 2; ++pair) {
-          if (pair && (mode == kBrickTracking || in_place || cells < 1024 || per > 2)) continue;
+          if (pair && (mode == kBrickTracking || in_place || geo.storage != kF32 || cells < 1024 || per > 2))
+            continue;
           const long long round = pair ? 2 * kBrickThreads : kBrickThreads;
           const double cell = mode == kBrickTracking ? 1.2e-3 : (cells >= 1024 && !pair ? 2.9e-3 : 2.7e-3);
           double work = 4.4e-4 * ((in_place ? phi / 3 : phi) + mu) + cell * ((cells + round - 1) / round * round);

@@ -680,9 +680,11 @@ const void* brick_kernel(int mode, int var, bool pair, bool in_place) {
                                   : LBM_BRICK_AA(kBrickCoupled, kVarSrtFlow | kVarD3Q7);
   }
 #undef LBM_BRICK_AA
-#define LBM_BRICK(MODE, VAR)                                            \
-  (pair ? reinterpret_cast<const void*>(&k_brick<MODE, VAR, S, 2>)      \
-        : reinterpret_cast<const void*>(&k_brick<MODE, VAR, S, 1>))
+// two cells per thread with FP32 populations only (brick_plan)
+#define LBM_BRICK(MODE, VAR)                                                       \
+  (pair && S == kF32 ? reinterpret_cast<const void*>(&k_brick<MODE, VAR, S, kPair>) \
+                     : reinterpret_cast<const void*>(&k_brick<MODE, VAR, S, 1>))
+  constexpr int kPair = S == kF32 ? 2 : 1;
   if (mode == kBrickTracking)
     return reinterpret_cast<const void*>(&k_brick<kBrickTracking, 0, S, 1>);
   switch (var) {

@@ -464,7 +464,6 @@ lbm_status plane_to_host(lbm_ctx* c, const float* dev, double* host, double* wid
     LBM_CK(c, lbm::launch_widen(dev, view, c->geo.n, c->stream));
     return LBM_OK;
   }
-  if (!wide) return fail(c, LBM_EINVAL, "read-out buffer changed from page-locked to pageable");
   LBM_CK(c, lbm::launch_widen(dev, wide, c->geo.n, c->stream));
   LBM_CK(c, cudaMemcpyAsync(host, wide, n * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   return LBM_OK;
