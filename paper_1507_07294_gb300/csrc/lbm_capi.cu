@@ -683,7 +683,11 @@ bool brick_applies(const lbm_ctx* c, int n) {
   if (n == 1 && c->geo.storage != lbm::kF32 && c->params.pattern == LBM_PATTERN_AB) return false;
   if (!bricks_have_room(c, n)) return false;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  return cudaStreamIsCapturing(c->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) {
+    cudaGetLastError();  // the default stream while another one captures: leave no error behind
+    return false;
+  }
+  return cap == cudaStreamCaptureStatusNone;
 }
 
 // n steps through the resident-brick kernel; with sums_out the sums of the state after them.
