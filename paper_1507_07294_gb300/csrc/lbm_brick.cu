@@ -17,8 +17,8 @@ cudaError_t state_sums_bf16(const float* state, const float* phi, const Geometry
 
 namespace {
 
-constexpr int kBrickPairLeast = 40000;      // bytes a block from which a third one matters
-constexpr int kBrickPairSmem = 77 * 1024;   // more than a third of an SM's 228 KB
+constexpr int kBrickTwoLeast = 54000;      // bytes a block from which a third one matters
+constexpr int kBrickTwoSmem = 77 * 1024;   // more than a third of an SM's 228 KB
 
 // ceil(2^kBrickDivShift / d), and whether k * it >> kBrickDivShift = k / d for every k up to
 // `most`.
@@ -153,9 +153,11 @@ BrickPlan brick_plan(const Geometry& geo, const Physics& ph, int mode, bool in_p
   // Two blocks an SM that leave shared memory for a third may be placed three on some SMs, and
   // the L1 cache, which the pulled f comes from several times, shrinks to what three leave: ask
   // for as much as lets no third in (97x105x57 52.2 -> 34.1 us a step, 83x117x63 48.2 -> 33.3,
-  // 128x110x43 40.6 -> 31.5; tracking 68x98x187 30.4 -> 24.9; unchanged below 480,000 cells).
-  if (p.nbricks > sms && p.nbricks <= 2 * sms && p.smem > kBrickPairLeast)
-    p.smem = std::max(p.smem, kBrickPairSmem);
+  // 128x110x43 40.6 -> 31.5; tracking 68x98x187 30.4 -> 24.9).  It counts from 54 KB a block (0.97
+  // of the time at 55 KB, 0.65 to 0.82 at 67 to 76; below it 0.99 to 1.01); with two cells per
+  // thread the registers keep a third out.
+  if (p.nbricks > sms && p.nbricks <= 2 * sms && !p.pair && p.smem > kBrickTwoLeast)
+    p.smem = std::max(p.smem, kBrickTwoSmem);
   const void* k = kernel_of(geo, ph, mode, p.pair != 0, in_place);
   int per = 0;
   if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kBrickSmem) != cudaSuccess ||
