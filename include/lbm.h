@@ -161,7 +161,7 @@ lbm_status lbm_init_phi(lbm_ctx* ctx, const double* phi, const double* u, const 
 lbm_status lbm_set_velocity(lbm_ctx* ctx, int kind, double U, double period);
 
 /* Advance n >= 0 time steps (Eqs. 4 and 20: stream, then collide in moment space with
- * Eqs. 17-18 and 31-32).  Asynchronous on the context's stream.  Small grids take all n
+ * Eqs. 17-18 and 31-32).  Asynchronous on the context's stream.  Small grids take up to 1024
  * steps in one kernel (see LBM_TUNE_BRICKS); on others pairs of steps are replayed from
  * CUDA graphs captured on first use (see LBM_TUNE_GRAPHS). */
 lbm_status lbm_step(lbm_ctx* ctx, int n);
@@ -289,9 +289,9 @@ lbm_status lbm_write_state(lbm_ctx* ctx, const float* f, const float* g,
  * it applies.  Identical results.
  * LBM_TUNE_BRICKS: 1 (default) lets lbm_step and lbm_step_reduce advance small grids
  * (up to 640,000 cells, 180,000 with 16-bit populations, 1.6 million in interface-tracking
- * mode; LBM_PATTERN_AA up to 36,000, 270,000 in interface-tracking mode) by one kernel per call that keeps every block on its own brick of
- * cells for all the steps, blocks waiting for their neighbours between steps.  The wait is
- * bounded by LBM_TUNE_TMA_WAIT_POLLS (to give the bricks another budget set that first, then
+ * mode; LBM_PATTERN_AA up to 36,000, 270,000 in interface-tracking mode) by one kernel for
+ * up to 1024 steps (interface tracking: 64) that keeps every block on its own brick of cells
+ * for all of them, blocks waiting for their neighbours between steps.  The wait is bounded by LBM_TUNE_TMA_WAIT_POLLS (to give the bricks another budget set that first, then
  * LBM_TUNE_BRICKS to 1); one that runs out is reported as LBM_ETIMEOUT like the TMA passes'
  * waits, and the steps since the last call that reported none are not valid.
  * lbm_get_tuning reports 1 only while it applies: not while profiling or with LBM_TUNE_FUSED,

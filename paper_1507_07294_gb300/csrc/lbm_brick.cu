@@ -76,6 +76,10 @@ bool divisions_ok(const AxisCut c[3], int halo) {
 // half as much each): 56x57x55 (176k cells) 14.4 -> 13.9 us, 64^3 (262k) 18.4 -> 18.5.  In
 // place a step has two waits and the bricks pay for the smallest boxes only: 32^3 9.2 -> 8.8
 // us, 48^3 11.3 -> 11.7; tracking 64^3 19.2 -> 12.4, 80^3 20.5 -> 21.0.
+// Boxes of any shape below the lines, part of the three-kernel step's time (geometric mean;
+// worst): FP32 0.87 (1.10 at 317x1049x1) over 110, FP16 0.77 (1.17 at 35x59x72) over 105; in
+// place FP32 0.86 (1.18 at 1x75x363) over 119, BF16 0.84 (1.14 at 33x29x22) over 109; tracking
+// in place 0.58 (0.88) over 81.
 long long brick_most_cells(int mode, int storage, bool in_place) {
   if (in_place) return mode == kBrickTracking ? 270000 : 36000;
   if (mode == kBrickTracking) return 1600000;
