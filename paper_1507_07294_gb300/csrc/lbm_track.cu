@@ -2,10 +2,10 @@
 // grids beyond the resident bricks: the order parameter (Eqs. 13, 16), the chemical potential
 // (Eq. 2) and the D3Q7 collision (Eqs. 15, 17, 18, 34) in one kernel, phi in shared memory
 // only.  The three passes move 128 B a cell (f twice, phi and mu written and read); this one
-// reads f and phi u once and writes them once, 80 B (75.6 by ncu at 192^3).  It is bound by
-// instruction issue and the barriers between planes, not by that traffic: 58 % of the issue
-// slots at 56 % of the DRAM rate.  Every value is formed by the operations of the three passes
-// in their order, so the state is the same bit for bit.
+// reads f and phi u once and writes them once, 80 B (78.6 by ncu at 192^3).  It is bound by
+// instruction issue and the barriers between planes, not by that traffic: 67 % of the issue
+// slots at 62 % of the DRAM rate, 395 instructions a cell.  Every value is formed
+// by the operations of the three passes in their order, so the state is the same bit for bit.
 // Measured per step, three passes -> one: 256^3 335 -> 282 us, 192^3 155 -> 128, 128^3
 // 55.4 -> 45.1 (k_track_rows); 150^3 91.8 -> 75.9, 200^3 193 -> 166 (k_track).
 #include <cuda_runtime.h>
