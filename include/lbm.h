@@ -331,8 +331,9 @@ lbm_status lbm_get_step(const lbm_ctx* ctx, long long* step);
 /* Per-kernel timing with CUDA events on the context's stream.  While enabled,
  * lbm_step brackets each kernel launch with events.  lbm_profile_read synchronises,
  * then returns for kernel k (0: order parameter, 1: chemical potential, 2: fused
- * stream-collide, or the single-pass step kernel where LBM_TUNE_FUSED applies) the
- * summed duration in ms and the number of launches since the last lbm_profile(ctx, 1). */
+ * stream-collide, or the kernel of the whole step where LBM_TUNE_FUSED applies or
+ * interface tracking takes one pass, which launch neither 0 nor 1) the summed duration in
+ * ms and the number of launches since the last lbm_profile(ctx, 1). */
 lbm_status lbm_profile(lbm_ctx* ctx, int enable);
 lbm_status lbm_profile_read(lbm_ctx* ctx, int kernel, double* total_ms,
                             long long* launches);

@@ -199,7 +199,8 @@ struct Sharers {
   std::map<const lbm_ctx*, Entry> live;
   std::atomic<unsigned> version{1};  // counts changes of `live`
 };
-Sharers g_sharers;
+// Never destroyed: a program may close contexts while it ends.
+Sharers& g_sharers = *new Sharers;
 
 // Sets or (part 0) takes back the part of the device that the context's bricks take.
 void share(lbm_ctx* c, double part) {
