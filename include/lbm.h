@@ -291,7 +291,8 @@ lbm_status lbm_write_state(lbm_ctx* ctx, const float* f, const float* g,
  * (up to 640,000 cells, 180,000 with 16-bit populations, 1.6 million in interface-tracking
  * mode; LBM_PATTERN_AA up to 36,000, 270,000 in interface-tracking mode) by one kernel for
  * up to 1024 steps (interface tracking: 64) that keeps every block on its own brick of cells
- * for all of them, blocks waiting for their neighbours between steps.  The wait is bounded by LBM_TUNE_TMA_WAIT_POLLS (to give the bricks another budget set that first, then
+ * for all of them, blocks waiting for their neighbours between steps; single tracking steps
+ * of more than 350,000 cells go without.  The wait is bounded by LBM_TUNE_TMA_WAIT_POLLS (to give the bricks another budget set that first, then
  * LBM_TUNE_BRICKS to 1); one that runs out is reported as LBM_ETIMEOUT like the TMA passes'
  * waits, and the steps since the last call that reported none are not valid.
  * lbm_get_tuning reports 1 only while it applies: not while profiling or with LBM_TUNE_FUSED,

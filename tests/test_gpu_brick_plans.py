@@ -32,3 +32,18 @@ def test_same_bits(L, shape, tracking):
             sa, sb = a.state(), b.state()
             for k in (0, 2) if tracking else (0, 1, 2):
                 assert np.array_equal(sa[k].view(np.uint32), sb[k].view(np.uint32))
+
+
+def test_single_tracking_steps_between_launches_of_many(L):
+    """Beyond 350,000 cells a single step is one pass over the box, several are bricks."""
+    w = I.perturbed(I.droplet(R=10.0, nx=75, ny=72, nz=70), seed=6, phi_amp=0.02)
+    w.velocity = ("deformation", 0.01, 40.0)
+    with L.Solver(w) as a, L.Solver(w, pattern="aa") as b:
+        L.lbm_set_tuning(b.ctx, L.LBM_TUNE_BRICKS, 0)
+        assert L.lbm_get_tuning(a.ctx, L.LBM_TUNE_BRICKS) == 1
+        for n in (1, 4, 1, 1, 3):
+            a.step(n)
+            b.step(n)
+            sa, sb = a.state(), b.state()
+            for k in (0, 2):
+                assert np.array_equal(sa[k].view(np.uint32), sb[k].view(np.uint32))
