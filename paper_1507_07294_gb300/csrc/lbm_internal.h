@@ -116,12 +116,13 @@ enum BrickMode { kBrickCoupled = 0, kBrickTracking = 1 };
 struct BrickPlan {
   int steps;
   int nbricks;      // 0: the grid does not go through the kernel
-  int slots;        // blocks that the device holds at once
   int mode, pair, in_place;
   int nb[3], b[3];  // bricks along each axis, cells of the largest along each axis
   int reach[3];     // bricks along each axis that lie within the cells a step reads
   int around;       // bricks a block waits for
   int smem;         // bytes of shared memory
+  int slots;        // blocks that the device holds at once; here the kernel is fastest: where the
+                    // members lie moves 32^3 by up to 7 % (4.94 us a step; 4.97 with it third)
   unsigned m_qx, m_qy, m_px, m_py, m_mx, m_my, m_bx, m_by;  // small_div of region sizes
 };
 struct BrickTimes {
