@@ -95,8 +95,8 @@ long long brick_most_cells(int mode, int storage, bool in_place) {
 // Two cells per thread pay from about 1024 cells a block (64x64x128, 256 bricks of 32x8x8:
 // 24.9 us, one cell per thread 26.3); they leave room for 2 blocks an SM instead of 3.  Boxes
 // with 16-bit populations are too small for that: none of 19,671 sampled ones took it.
-// Measured per step, three passes -> bricks: 16^3 9.2 -> 4.2 us, 32^3 9.2 -> 5.1, 48^3
-// 11.5 -> 7.9, 64^3 18.5 -> 13.9, 64x64x128 29.6 -> 25.1, 37x41x45 10.3 -> 8.5; tracking 48^3
+// Measured per step, three passes -> bricks: 16^3 9.2 -> 4.2 us, 32^3 9.2 -> 4.9, 48^3
+// 11.5 -> 7.9, 64^3 18.5 -> 13.7, 64x64x128 29.6 -> 25.1, 37x41x45 10.3 -> 8.5; tracking 48^3
 // 12.3 -> 5.6, 100^3 30.6 -> 21.3; FP16 32^3 10.2 -> 6.2.
 BrickPlan brick_plan(const Geometry& geo, const Physics& ph, int mode, bool in_place, int sms) {
   BrickPlan p{};

@@ -16,9 +16,9 @@
 // Every value is formed by the operations of the three passes in their order, so the state
 // is the same bit for bit.
 //
-// At 32^3 a step's 5.1 us are the wait (0.6), the loads' issue (0.5), phi
+// At 32^3, when a step took 5.1 us (4.9 now), these were the wait (0.6), the loads' issue (0.5), phi
 // (0.9), mu (0.5), the collision (1.4) and the release of the stores (0.6), as clocks read
-// in the kernel say: latency throughout.  At 64^3 (13.9 us) the collision's
+// in the kernel say: latency throughout.  At 64^3 (13.7 us) the collision's
 // arithmetic is the largest part.  brick_plan has the times over the sizes.
 #pragma once
 
